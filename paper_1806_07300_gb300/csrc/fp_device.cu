@@ -82,11 +82,13 @@ int scratch_alloc(int device, void **out, size_t bytes, cudaStream_t s) {
     return FP_OK;
 }
 
-// rows tile (feature-major) + nbuf bin blocks + votes + per-warp task rings
+// bytes of a slab: 32 rows of F features and C counters (none for leaf ids)
+size_t slab_bytes(int F, int C, bool leaves) { return 128 * ((size_t)F + (leaves ? 0 : C)); }
+
+// the tile's slabs + nbuf bin blocks + per-warp task rings (R is a multiple of 32)
 size_t smem_bytes(int R, int F, int head_smem, int nbuf, int C, int warps, bool leaves) {
-    const size_t xs = ((size_t)R * F * 4 + 15) & ~(size_t)15;
-    const size_t votes = leaves ? 0 : (((size_t)R * C * 4 + 15) & ~(size_t)15);
-    return xs + (size_t)nbuf * (size_t)head_smem + votes + (size_t)warps * FP_RING * 8;
+    return (size_t)(R / 32) * slab_bytes(F, C, leaves) + (size_t)nbuf * (size_t)head_smem +
+           (size_t)warps * FP_RING * 8;
 }
 
 // The kernel variant for a forest and block size: its kind of super-node
@@ -94,7 +96,8 @@ size_t smem_bytes(int R, int F, int head_smem, int nbuf, int C, int warps, bool 
 // for several CTAs per SM (<= 42 registers), larger blocks the one-CTA build ...
 template <int MODE, int DK, int HK>
 void (*traverse_kernel_sized(const fp_device_forest *f))(TravParams) {
-    return f->threads <= 768 ? fp_traverse_kernel<MODE, 2, DK, HK> : fp_traverse_kernel<MODE, 1, DK, HK>;
+    if (f->hdr.n_super == 0) return fp_traverse_kernel<MODE, 1, DK, HK, true>;  // one build serves every CTA size
+    return f->threads <= 768 ? fp_traverse_kernel<MODE, 2, DK, HK, false> : fp_traverse_kernel<MODE, 1, DK, HK, false>;
 }
 
 // ... and its head kind (compiled in: 0 ranked, 1 level slots, 2 paired).
@@ -249,6 +252,7 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
     const int64_t want = (n * std::max<int32_t>(1, h.n_passes) + grid - 1) / grid;  // rows per tile
     if (want < R) R = (int32_t)std::max<int64_t>(32, (want + 31) / 32 * 32);
     p.R = R;
+    p.slab = (uint32_t)slab_bytes(h.n_features, h.n_classes, false);  // other modes set their own
     p.n_tiles = (n + R - 1) / R;
     p.head_smem = f->head_smem;
     p.nbuf = f->nbuf;
@@ -260,12 +264,16 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
     p.status = f->d_status;
     p.spin_limit = f->spin_limit;
     p.stall = f->stall;
-    p.n_super = h.n_super;
+    p.n_super = (uint32_t)h.n_super;
     p.deep_kind = deep_kind(h);
     if (p.deep_kind >= 3) {
-        p.fbits = (uint32_t)h.feature_bits;
-        p.cbits = (uint32_t)h.class_bits;
-        p.sh2 = (p.deep_kind == 4 ? 1 : 2) * p.fbits + 2 * p.cbits;
+        const uint32_t fb = (uint32_t)h.feature_bits, cb = (uint32_t)h.class_bits;
+        p.cshl = (p.deep_kind == 4 ? 1 : 2) * fb;
+        p.cshr = p.cshl + cb;
+        p.tie = 1u << (p.cshr + cb);
+        p.frot = (fb + 25u) & 31u;  // right by fb - 7
+        p.fmask = (1u << fb) - 1u;
+        p.cmask = (1u << cb) - 1u;
         p.klo = h.key_lo;
         p.khi = h.key_hi;
         p.kshl = h.key_shl;
@@ -273,8 +281,6 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
         p.kga = h.key_gap_a;
         p.kgb = h.key_gap_b;
         p.kgd = h.key_gap_d;
-        p.fmask = (1u << p.fbits) - 1u;
-        p.cmask = (1u << p.cbits) - 1u;
         p.vbase3 = (uint32_t)h.values3_base;
         p.deep_keys = reinterpret_cast<const uint32_t *>(f->d_image + h.off_deep_keys);
     }
@@ -325,6 +331,14 @@ extern "C" int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_for
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemsetAsync"); goto fail; }
     e = cudaMemcpyAsync(f->d_image, img, (size_t)h->total_bytes, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMemcpyAsync(image)"); goto fail; }
+    if (h->n_values > 0 && h->n_super == 0) {
+        fp_inline_values_kernel<<<(unsigned)h->n_bins, 256, 0, s>>>(
+            f->d_image + h->off_heads, reinterpret_cast<const FpBin *>(f->d_image + h->off_bins),
+            reinterpret_cast<const float *>(f->d_image + h->off_values), (uint32_t)h->n_values,
+            h->head_select == 2 ? 16u : 8u);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) { rc = cuda_fail(e, "fp_inline_values_kernel launch"); goto fail; }
+    }
     e = cudaStreamSynchronize(s);  // the caller may free the host image on return
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaStreamSynchronize"); goto fail; }
     f->head_smem = (h->max_head_bytes + 15) & ~15;
@@ -428,6 +442,7 @@ extern "C" int fp_predict_values(const fp_device_forest *f, const float *X, int6
     TravParams p = base_params(f, X, n);
     p.n_passes = h.n_passes;
     p.n_items = p.n_tiles * h.n_passes;
+    p.slab = (uint32_t)slab_bytes(h.n_features, 1, false);
     p.vscale = scale;
     p.vbias = bias;
     p.out_val = out;
@@ -548,6 +563,7 @@ extern "C" int fp_predict_leaves(const fp_device_forest *f, const float *X, int6
     TravParams p = base_params(f, X, n);
     p.n_passes = f->hdr.n_passes;
     p.n_items = p.n_tiles * f->hdr.n_passes;
+    p.slab = (uint32_t)slab_bytes(f->hdr.n_features, 0, true);
     p.out_leaf = out_leaf;
     const int64_t grid = std::min<int64_t>(p.n_items, f->grid_leaves);
     traverse_kernel<FP_MODE_LEAVES>(f)<<<(unsigned)grid, f->threads, f->smem_leaves, s>>>(p);

@@ -5,27 +5,33 @@
 // resident in L2 while every tile of observations goes through them (the GPU
 // counterpart of the paper's bins bound to cores, Section III).  For an item
 // the CTA:
-//   1. stages the tile's rows into shared memory feature-major
-//      (x[f * R + r]), so 32 lanes holding 32 consecutive rows read any
-//      features from 32 different banks (16-byte loads along a row when the
-//      feature count is a multiple of 4, else 4-byte cp.async); for a forest
-//      with three-level super-nodes each value is turned into its order key
-//      (fp_internal.h) and every compare is an unsigned integer compare,
-//      otherwise values and compares stay float;
+//   1. stages the tile's rows into shared memory in slabs of 32 rows: a slab
+//      holds its F features and then its vote counters (one per class, or one
+//      float sum), 32 words each, row l of the slab in column l.  32 lanes
+//      holding the 32 rows of a slab read any features and count any votes in
+//      32 different banks, and feature f of a row is 128 * f bytes past the
+//      row's own address, so a task carries that one address and no step
+//      multiplies by the tile size.  For a forest with three-level
+//      super-nodes each value is turned into its order key (fp_internal.h)
+//      and every compare is an unsigned integer compare, otherwise values and
+//      compares stay float;
 //   2. streams the bins' interleaved blocks (the heads of their trees,
 //      Section III-A Bin) through nbuf (2 or 3) shared-memory buffers with TMA bulk
 //      copies (cp.async.bulk) completing on mbarriers: a warp waits only for
-//      the block of the bin it is about to claim, and the last warp to finish
-//      claiming a bin refills that buffer with the bin nbuf places ahead;
+//      the block of the bin it walks next, and the last warp done with a
+//      bin's block refills that buffer with the bin nbuf places ahead;
 //   3. walks (observation, tree) tasks in two kinds of warp steps:
-//        burst -- the warp claims 32 consecutive tasks (32 rows of one tree)
-//                 and all lanes walk their paths through the tree's head in
-//                 shared memory together, with a branch-free step (level
-//                 heads: exactly d+1 steps over implicit slots, or (d+1)/2
-//                 steps of two levels when the slots are paired; ranked
-//                 heads: until the last lane leaves the head); paths that leave the
-//                 head are pushed, compacted with __ballot_sync / __popc,
-//                 into the warp's ring of pending tasks;
+//        burst -- the warp takes its next unit, the 32 rows of one slab and
+//                 one tree, and all lanes walk their paths through the tree's
+//                 head in shared memory together, with a branch-free step
+//                 (level heads: exactly d+1 steps over implicit slots, or
+//                 (d+1)/2 steps of two levels when the slots are paired;
+//                 ranked heads: until the last lane leaves the head); paths
+//                 that leave the head are pushed, compacted with
+//                 __ballot_sync / __popc, into the warp's ring of pending
+//                 tasks.  Units are claimed from a shared counter: dealt out
+//                 to the warps in turn they cost no atomic, but the slowest
+//                 warp then held up each bin's buffer, 8 % of the run;
 //        deep  -- every lane holding a task resolves two or three more levels
 //                 with one 32-byte super-node load (one L2 sector); a lane
 //                 that reaches a leaf votes and takes the next pending task
@@ -46,7 +52,15 @@
 // writes bias + scale * sum (several passes: summed in global memory, the
 // last pass's CTA writes it).
 //
-// Waits: cp.async.wait_group and __syncthreads are hardware waits; a wait for
+// What bounds it (256 trees of 78.8k nodes, 28 features, 4 M rows, bins of 5
+// trees with heads 0..9: 25.4 ms, 27.5 ms before steps were straight-line code
+// over slabs): the load/store data pipe, 77 % busy with 6.1 wavefronts per
+// (row, tree), about half of them the super-nodes' sectors and half
+// shared-memory words; 19.8 warp instructions per (row, tree) (23.4 before)
+// take 62 % of the issue slots, the ALU pipe being the busiest of the
+// arithmetic ones.
+//
+// Waits: __syncthreads is a hardware wait; a wait for
 // a bin block polls its mbarrier at most spin_limit times (FP_SPIN_LIMIT
 // unless a test lowers it), then records FP_ETIMEOUT in the status word and
 // makes every warp skip the rest of its work; before exiting, the CTA waits
@@ -71,6 +85,7 @@ struct TravParams {
     int64_t n_tiles;
     int64_t n_items;
     int32_t F, C, T, R;
+    uint32_t slab;            // bytes of a slab: 32 rows of F features and the mode's counters
     int32_t n_passes;
     int32_t head_smem;        // bytes reserved for one bin block
     int32_t nbuf;             // bin-block buffers (2 or 3)
@@ -91,14 +106,16 @@ struct TravParams {
     int32_t spin_limit;       // polls of a bin block's barrier before the wait gives up
     int32_t stall;            // fault injection: bin waits ignore completed copies (0 normally)
     int32_t deep_kind;        // super-nodes: 2 two levels, 3 three levels (format 1), 4 three levels (format 2)
-    uint32_t fbits, sh2;      // three levels: feature bits; key-prefix shift of the last level
-                              // (2fb + 2cb in format 1, fb + 2cb in format 2)
-    uint32_t cbits, fmask, cmask;  // three levels: class bits, feature and class masks
+    uint32_t tie;             // three levels: equal key prefixes of the last level differ only below this
+                              // (2fb + 2cb bits in format 1, fb + 2cb in format 2)
+    uint32_t frot;            // format 1: rotation that brings an upper slot's feature to bit 7
+    uint32_t cshl, cshr;      // three levels: where a last-level word holds its left and right exits' classes
+    uint32_t fmask, cmask;    // three levels: feature and class masks
     uint32_t vbase3;          // three levels, values mode: first per-exit value slot
     const uint32_t *deep_keys;  // three levels: full keys, 4 (format 1) or 8 (format 2) per super-node
     uint32_t klo, khi, kshl, kflag;  // format 2: the key remap V of the staged rows
     uint32_t kga, kgb, kgd;          // format 2: its collapsed run of keys
-    int64_t n_super;
+    uint32_t n_super;         // super-nodes (below 2^31)
 };
 
 // What a kernel computes per (row, tree) task it finishes.
@@ -112,31 +129,21 @@ struct TravParams {
 #define FP_SPIN_LIMIT (1 << 24)
 #define FP_RING 64            // pending tasks per warp
 #define FP_NO_CLASS (FP_REF_LEAF | 0x7FFFFFFFu)
+#define FP_NO_TASK 0xFFFFFFFFu  // a lane's ref when it holds no task (super-node indices are below 2^31)
 
-__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
-    uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    uint32_t s = (uint32_t)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
-
-// One super-node: a single 256-bit load (32-byte aligned, one L2 sector).
+// One super-node: a single 256-bit load (32-byte aligned, one L2 sector), for
+// the lanes that hold a task (ref is no index otherwise).
 // The lines are not allocated in L1: few super-nodes are read twice by one
 // SM before eviction, and with most of the unified L1/shared array given to
 // shared memory, allocating a line per lane for thousands of loads in
 // flight throttles the load path (measured: twice the run time once shared
 // memory takes more than about 196 KB).  The memory clobber keeps the load
 // where it is written, ahead of the work meant to overlap its latency.
-__device__ __forceinline__ void ld_super(const FpSuper *p, uint32_t w[8]) {
-    asm volatile("ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
-                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-                 : "l"(p)
+__device__ __forceinline__ void ld_super(const FpSuper *deep, uint32_t ref, uint32_t w[8]) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %9, %10;\n"
+                 " @p ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n}\n"
+                 : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]), "+r"(w[6]), "+r"(w[7])
+                 : "l"(deep + ref), "r"(ref), "n"(FP_NO_TASK)
                  : "memory");
 }
 
@@ -205,94 +212,154 @@ __device__ __forceinline__ void stage_block_bulk(const TravParams &p, int b, uin
         : "memory");
 }
 
-// Per-lane state of a running task.
-struct LaneTask {
-    bool active;
-    int r;            // row within the tile
-    int t;            // tree
-    uint32_t ref;     // current super-node (index into deep)
+// CTA-wide state shared by the items a CTA runs.
+struct CtaShared {
+    uint64_t full[FP_NBUF];   // block staged (bulk copy done)
+    int next[FP_NBUF];        // next untaken unit of the buffer's bin
+    int done[FP_NBUF];        // warps done with the buffer's bin
+    int issued[FP_NBUF];      // bulk copies issued into the buffer
+    uint32_t phases;          // parities of issued[] when the current item started
+    int bin0, bin1;           // the current item's bins
+    int64_t tile;             // the current item's tile
+    int last;
+    int abort;
+    long long next_item;
 };
 
-// A finished task: vote, record the leaf id (parity mode) or add the leaf's
-// value to the row's sum (cls is then the leaf's value slot).
+// A word of dynamic shared memory at a byte offset, by its 32-bit address
+// (through a pointer the walks took 5 to 9 % longer).
+__device__ __forceinline__ uint32_t lds(const uint8_t *smem, uint32_t off) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(smem_u32(smem) + off));
+    return v;
+}
+
+__device__ __forceinline__ uint4 lds128(const uint8_t *smem, uint32_t off) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "r"(smem_u32(smem) + off));
+    return v;
+}
+
+// Per-lane state of a running task.  A corrupt record only sets `bad`,
+// reported at the item's end, so that a step stays straight-line code.
+struct LaneTask {
+    uint32_t ref;     // current super-node (index into deep), or FP_NO_TASK
+    uint32_t xb;      // shared-memory offset of the row: feature f is 128 f bytes further on
+    uint32_t rt;      // parity mode: row within the tile | tree << 11
+    int bad;
+};
+
+// A finished task's memory read whose result is not used at once: the leaf's
+// value on its way to the row's sum (values mode), or its leaf id on its way
+// to the output (parity mode).  Used one step later, when it has arrived; a
+// use at once stalls the warp for a whole L2 latency in nearly every step.
+struct Pending {
+    bool on;
+    uint32_t at;      // values: xb; parity: rt
+    uint32_t word;
+};
+
+// A vote for class `cls` of the row at xb.  Class 0 is not counted: its votes
+// are the item's trees less all the others'.  Returns false for a class that
+// does not exist.
+__device__ __forceinline__ bool vote(const TravParams &p, uint8_t *smem, bool on, uint32_t xb, uint32_t cls) {
+    const bool counted = cls - 1u < (uint32_t)p.C - 1u;
+    if (on && counted) atomicAdd(reinterpret_cast<uint32_t *>(smem + xb + (((uint32_t)p.F + cls) << 7)), 1u);
+    return !on || counted || cls == 0u;
+}
+
+// The row's sum of leaf values (values mode).
+__device__ __forceinline__ void add_value(const TravParams &p, uint8_t *smem, uint32_t xb, float v) {
+    atomicAdd(reinterpret_cast<float *>(smem + xb + ((uint32_t)p.F << 7)), v);
+}
+
+__device__ __forceinline__ void put_leaf(const TravParams &p, const CtaShared &sh, uint32_t rt, int32_t leaf_id) {
+    p.out_leaf[(sh.tile * p.R + (rt & 2047u)) * p.T + (rt >> 11)] = leaf_id;
+}
+
 template <int MODE>
-__device__ __forceinline__ void finish(const TravParams &p, uint32_t *svotes, int64_t row0, int r, int t,
-                                       uint32_t cls, int32_t leaf_id) {
-    if (MODE == FP_MODE_LEAVES) {
-        p.out_leaf[(row0 + r) * p.T + t] = leaf_id;
-    } else if (MODE == FP_MODE_VALUES) {
-        if (cls < p.n_vals)
-            atomicAdd(reinterpret_cast<float *>(svotes) + r, __ldg(p.leaf_val + cls));
+__device__ __forceinline__ void settle(const TravParams &p, uint8_t *smem, const CtaShared &sh, Pending &pend) {
+    if (MODE == FP_MODE_VOTES) return;
+    if (pend.on) {
+        if (MODE == FP_MODE_VALUES)
+            add_value(p, smem, pend.at, __uint_as_float(pend.word));
         else
-            report(p.status, FP_ERR_FLAG_DEVICE);
-    } else if (cls < (uint32_t)p.C) {
-        atomicAdd(&svotes[cls * p.R + r], 1u);  // class-major: a burst's 32 rows hit 32 banks
-    } else {
-        report(p.status, FP_ERR_FLAG_DEVICE);
+            put_leaf(p, sh, pend.at, (int32_t)pend.word);
     }
+    pend.on = false;
 }
 
 // Lanes without a task take pending ones from the warp's ring.
+template <int MODE>
 __device__ __forceinline__ void pop_tasks(const TravParams &p, const uint2 *ring, int &head, int tail, LaneTask &L,
                                           unsigned lt_mask) {
-    const unsigned idle = __ballot_sync(0xffffffffu, !L.active);
-    const int npop = min(__popc(idle), tail - head);
-    if (npop <= 0) return;
+    const bool free = L.ref == FP_NO_TASK;
+    const unsigned idle = __ballot_sync(0xffffffffu, free);
     const int rk = __popc(idle & lt_mask);
-    if (!L.active && rk < npop) {
+    if (free && rk < tail - head) {
         const uint2 ent = ring[(head + rk) & (FP_RING - 1)];
         L.ref = ent.x;
-        L.r = (int)(ent.y & 2047u);
-        L.t = (int)(ent.y >> 11);
-        L.active = true;
-    }
-    head += npop;
-}
-
-// One deep step, two or three levels of the tree per 32-byte load, in two
-// halves: the load is issued first and consumed after the warp has done other
-// work (a head burst), so the L2 latency overlaps that work.
-__device__ __forceinline__ void deep_issue(const TravParams &p, const LaneTask &L, uint32_t w[8]) {
-    ld_super(p.deep + L.ref, w);
-}
-
-// Three levels: full keys for the first two, and a key prefix for the last,
-// whose tie (rare) is decided by the slot's full key from the side table.
-template <int MODE>
-__device__ __forceinline__ void deep_finish3(const TravParams &p, const uint32_t *xs, uint32_t *svotes, int64_t row0,
-                                             LaneTask &L, const uint32_t w[8]) {
-    const uint32_t *xr = xs + L.r;
-    const int R = p.R;
-    const uint32_t fm = p.fmask, fb = p.fbits, s2 = p.sh2;
-    const uint32_t k0 = xr[((w[3] >> fb) & fm) * R];
-    const uint32_t d0 = k0 > w[0] ? 1u : 0u;
-    const uint32_t n1 = d0 ? w[2] : w[1];
-    const uint32_t k1 = xr[(((d0 ? w[5] : w[4]) >> fb) & fm) * R];
-    const uint32_t d1 = k1 > n1 ? 1u : 0u;
-    const uint32_t j = 2 * d0 + d1;  // last-level slot 3 + j
-    const uint32_t n2 = d0 ? (d1 ? w[6] : w[5]) : (d1 ? w[4] : w[3]);
-    const uint32_t k2 = xr[(n2 & fm) * R];
-    uint32_t d2 = (k2 >> s2) > (n2 >> s2) ? 1u : 0u;
-    if ((k2 >> s2) == (n2 >> s2)) d2 = k2 > __ldg(p.deep_keys + 4 * (int64_t)L.ref + j) ? 1u : 0u;
-    const uint32_t e = 2 * j + d2;
-    const uint32_t mask = w[7] >> 24;
-    if ((mask >> e) & 1u) {
-        L.active = false;
-        int32_t leaf_id = -1;
-        if (MODE == FP_MODE_LEAVES) leaf_id = p.deep_leaf[8 * (int64_t)L.ref + e];
-        const uint32_t cls =
-            MODE == FP_MODE_VALUES ? p.vbase3 + 8 * L.ref + e : (n2 >> (2 * fb + p.cbits * d2)) & p.cmask;
-        finish<MODE>(p, svotes, row0, L.r, L.t, cls, leaf_id);
-    } else {
-        // children sit side by side from the offset on, in exit order
-        const uint32_t nref = L.ref + (w[7] & FP_DEEP3_OFFSET_MASK) + __popc(~mask & ((1u << e) - 1u));
-        if (nref > L.ref && (int64_t)nref < p.n_super) {  // forward only, so every walk ends
-            L.ref = nref;
+        if (MODE == FP_MODE_LEAVES) {
+            L.rt = ent.y;
+            L.xb = ((ent.y & 2047u) >> 5) * p.slab + (ent.y & 31u) * 4u;
         } else {
-            report(p.status, FP_ERR_FLAG_DEVICE);
-            L.active = false;
+            L.xb = ent.y;
         }
     }
+    head = min(head + __popc(idle), tail);
+}
+
+// One deep step in two halves: the load is issued first and consumed after
+// the warp has done other work (a head burst), so the L2 latency overlaps
+// that work.  The second half is written without branches (but for key ties,
+// which are rare): all lanes compute, and the lanes without a task keep
+// nothing.  Its outcome:
+struct DeepStep {
+    bool leaf;
+    uint32_t cls;         // the leaf's class (two levels, values mode: its value slot)
+    uint32_t next;        // the next super-node
+    uint32_t e;           // the exit taken
+};
+
+// Three levels: exit e is a leaf, or leads to one of the super-node's
+// children, which sit side by side from the offset on, in exit order.
+__device__ __forceinline__ void exit3(uint32_t ref, uint32_t w7, DeepStep &s) {
+    // bit 24: exit e leads on; below it: the exits before e that lead on
+    const uint32_t on = (~w7 & 0xFF000000u) >> s.e;
+    s.leaf = (on & (1u << 24)) == 0u;
+    s.next = ref + (w7 & FP_DEEP3_OFFSET_MASK) + __popc(on & 0xFFFFFFu);
+}
+
+// Three levels, format 1: full keys for the first two, and a key prefix for
+// the last, whose tie (rare) is decided by the slot's full key from the side
+// table.
+__device__ __forceinline__ DeepStep deep_step3(const TravParams &p, const uint8_t *smem, uint32_t ref, uint32_t xb,
+                                               const uint32_t w[8]) {
+    const uint32_t fm7 = p.fmask << 7;
+    const uint32_t k0 = lds(smem, xb + (__funnelshift_r(w[3], w[3], p.frot) & fm7));
+    const bool r0 = k0 > w[0];
+    const uint32_t n1 = r0 ? w[2] : w[1], m1 = r0 ? w[5] : w[4];
+    const uint32_t k1 = lds(smem, xb + (__funnelshift_r(m1, m1, p.frot) & fm7));
+    const bool r1 = k1 > n1;
+    const uint32_t n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
+    const uint32_t k2 = lds(smem, xb + ((n2 & p.fmask) << 7));
+    bool r2 = k2 > n2;  // decided by the key bits, unless they are equal
+    DeepStep s;
+    s.e = (r0 ? 4u : 0u) + (r1 ? 2u : 0u);
+    // behind a vote, so that the steps without a tie issue no load of the side
+    // table; predicated off in every lane it still takes the load/store pipe
+    // a wavefront a step (2 % of the run)
+    const bool tie = (k2 ^ n2) < p.tie && ref != FP_NO_TASK;
+    if (__any_sync(0xffffffffu, tie)) {
+        if (tie) r2 = k2 > __ldg(p.deep_keys + 4 * (int64_t)ref + (s.e >> 1));
+        __syncwarp();
+    }
+    s.e += r2 ? 1u : 0u;
+    s.cls = (n2 >> (r2 ? p.cshr : p.cshl)) & p.cmask;
+    exit3(ref, w[7], s);
+    return s;
 }
 
 // Three levels, format 2: every slot's word is the top bits of its remapped
@@ -300,96 +367,212 @@ __device__ __forceinline__ void deep_finish3(const TravParams &p, const uint32_t
 // whole word decides the split wherever their top bits differ.  Where they
 // are equal for any of the three slots of the walk (rare), the step is taken
 // again with the slots' full keys from the side table.
-template <int MODE>
-__device__ __forceinline__ void deep_finish3p(const TravParams &p, const uint32_t *xs, uint32_t *svotes,
-                                              int64_t row0, LaneTask &L, const uint32_t w[8]) {
-    const uint32_t *xr = xs + L.r;
-    const int R = p.R;
-    const uint32_t fm = p.fmask, fb = p.fbits, s2 = p.sh2;
-    const uint32_t k0 = xr[(w[0] & fm) * R];
-    uint32_t d0 = k0 > w[0] ? 1u : 0u;
-    uint32_t n1 = d0 ? w[2] : w[1];
-    const uint32_t k1 = xr[(n1 & fm) * R];
-    uint32_t d1 = k1 > n1 ? 1u : 0u;
-    uint32_t j = 2 * d0 + d1;  // last-level slot 3 + j
-    uint32_t n2 = d0 ? (d1 ? w[6] : w[5]) : (d1 ? w[4] : w[3]);
-    uint32_t k2 = xr[(n2 & fm) * R];
-    uint32_t d2 = k2 > n2 ? 1u : 0u;
-    if ((min(k0 ^ w[0], k1 ^ n1) >> fb) == 0u || ((k2 ^ n2) >> s2) == 0u) {
-        const uint32_t *fk = p.deep_keys + 8 * (int64_t)L.ref;
-        d0 = k0 > __ldg(fk) ? 1u : 0u;
-        n1 = d0 ? w[2] : w[1];
-        d1 = xr[(n1 & fm) * R] > __ldg(fk + 1 + d0) ? 1u : 0u;
-        j = 2 * d0 + d1;
-        n2 = d0 ? (d1 ? w[6] : w[5]) : (d1 ? w[4] : w[3]);
-        k2 = xr[(n2 & fm) * R];
-        d2 = k2 > __ldg(fk + 3 + j) ? 1u : 0u;
-    }
-    const uint32_t e = 2 * j + d2;
-    const uint32_t mask = w[7] >> 24;
-    if ((mask >> e) & 1u) {
-        L.active = false;
-        int32_t leaf_id = -1;
-        if (MODE == FP_MODE_LEAVES) leaf_id = p.deep_leaf[8 * (int64_t)L.ref + e];
-        const uint32_t cls =
-            MODE == FP_MODE_VALUES ? p.vbase3 + 8 * L.ref + e : (n2 >> (fb + p.cbits * d2)) & p.cmask;
-        finish<MODE>(p, svotes, row0, L.r, L.t, cls, leaf_id);
-    } else {
-        const uint32_t nref = L.ref + (w[7] & FP_DEEP3_OFFSET_MASK) + __popc(~mask & ((1u << e) - 1u));
-        if (nref > L.ref && (int64_t)nref < p.n_super) {  // forward only, so every walk ends
-            L.ref = nref;
-        } else {
-            report(p.status, FP_ERR_FLAG_DEVICE);
-            L.active = false;
+__device__ __forceinline__ DeepStep deep_step3p(const TravParams &p, const uint8_t *smem, uint32_t ref, uint32_t xb,
+                                                const uint32_t w[8]) {
+    const uint32_t fm = p.fmask;
+    const uint32_t k0 = lds(smem, xb + ((w[0] & fm) << 7));
+    bool r0 = k0 > w[0];
+    uint32_t n1 = r0 ? w[2] : w[1];
+    const uint32_t k1 = lds(smem, xb + ((n1 & fm) << 7));
+    bool r1 = k1 > n1;
+    uint32_t n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
+    uint32_t k2 = lds(smem, xb + ((n2 & fm) << 7));
+    bool r2 = k2 > n2;
+    // one test for the three slots, by the last level's shorter prefix: it
+    // takes a few more steps again than need be
+    const bool tie = min(min(k0 ^ w[0], k1 ^ n1), k2 ^ n2) < p.tie && ref != FP_NO_TASK;
+    if (__any_sync(0xffffffffu, tie)) {
+        if (tie) {
+            const uint32_t *fk = p.deep_keys + 8 * (int64_t)ref;
+            r0 = k0 > __ldg(fk);
+            n1 = r0 ? w[2] : w[1];
+            r1 = lds(smem, xb + ((n1 & fm) << 7)) > __ldg(fk + 1 + (r0 ? 1 : 0));
+            n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
+            k2 = lds(smem, xb + ((n2 & fm) << 7));
+            r2 = k2 > __ldg(fk + 3 + (r0 ? 2 : 0) + (r1 ? 1 : 0));
         }
+        __syncwarp();
     }
+    DeepStep s;
+    s.e = (r0 ? 4u : 0u) + (r1 ? 2u : 0u) + (r2 ? 1u : 0u);
+    s.cls = (n2 >> (r2 ? p.cshr : p.cshl)) & p.cmask;
+    exit3(ref, w[7], s);
+    return s;
+}
+
+// Two levels, float thresholds.
+__device__ __forceinline__ DeepStep deep_step2(const uint8_t *smem, uint32_t xb, const uint32_t w[8]) {
+    const bool r0 = !goes_left<false>(lds(smem, xb + ((w[3] & 1023u) << 7)), w[0]);
+    const uint32_t f1 = r0 ? (w[3] >> 20) & 1023u : (w[3] >> 10) & 1023u;
+    const bool r1 = !goes_left<false>(lds(smem, xb + (f1 << 7)), r0 ? w[2] : w[1]);
+    const uint32_t x = r0 ? (r1 ? w[7] : w[6]) : (r1 ? w[5] : w[4]);
+    DeepStep s;
+    s.leaf = (x & FP_REF_LEAF) != 0u;
+    s.cls = x & 0x7FFFFFFFu;
+    s.next = x;
+    s.e = (r0 ? 2u : 0u) + (r1 ? 1u : 0u);
+    return s;
 }
 
 // DK: the forest's kind of super-node (p.deep_kind: 2, 3 or 4); a
 // compile-time choice, so no kind's step carries another's code.
 template <int MODE, int DK>
-__device__ __forceinline__ void deep_finish(const TravParams &p, const uint32_t *xs, uint32_t *svotes, int64_t row0,
-                                            LaneTask &L, const uint32_t w[8]) {
-    if (DK == 3) {
-        deep_finish3<MODE>(p, xs, svotes, row0, L, w);
-        return;
+__device__ __forceinline__ void deep_finish(const TravParams &p, uint8_t *smem, LaneTask &L, Pending &pend,
+                                            const uint32_t w[8]) {
+    const uint32_t ref = L.ref;
+    const bool on = ref != FP_NO_TASK;
+    const DeepStep s = DK == 3   ? deep_step3(p, smem, ref, L.xb, w)
+                       : DK == 4 ? deep_step3p(p, smem, ref, L.xb, w)
+                                 : deep_step2(smem, L.xb, w);
+    const bool leaf = on && s.leaf;
+    if (MODE == FP_MODE_VOTES) {
+        const uint32_t c1 = s.cls - 1u, nc = (uint32_t)p.C - 1u;
+        if (leaf && c1 < nc) atomicAdd(reinterpret_cast<uint32_t *>(smem + L.xb + (((uint32_t)p.F + s.cls) << 7)), 1u);
+        if (leaf && s.cls > nc) L.bad = 1;
+    } else if (MODE == FP_MODE_VALUES) {  // start the read of the leaf's value ...
+        const uint32_t slot = DK == 2 ? s.cls : p.vbase3 + 8 * ref + s.e;
+        const bool ok = slot < p.n_vals;
+        L.bad |= leaf && !ok;
+        if (leaf && ok) {
+            pend.on = true;
+            pend.at = L.xb;
+            pend.word = __float_as_uint(__ldg(p.leaf_val + slot));
+        }
+    } else if (leaf) {  // ... or of its id
+        pend.on = true;
+        pend.at = L.rt;
+        pend.word = (uint32_t)__ldg(p.deep_leaf + (DK == 2 ? 4 : 8) * (int64_t)ref + s.e);
     }
-    if (DK == 4) {
-        deep_finish3p<MODE>(p, xs, svotes, row0, L, w);
-        return;
-    }
-    const int R = p.R;
-    const uint32_t x0 = xs[(w[3] & 1023u) * R + L.r];
-    const uint32_t d0 = goes_left<false>(x0, w[0]) ? 0u : 1u;
-    const uint32_t f1 = d0 ? (w[3] >> 20) & 1023u : (w[3] >> 10) & 1023u;
-    const uint32_t t1 = d0 ? w[2] : w[1];
-    const uint32_t x1 = xs[f1 * R + L.r];
-    const uint32_t d1 = goes_left<false>(x1, t1) ? 0u : 1u;
-    const uint32_t nref = d0 ? (d1 ? w[7] : w[6]) : (d1 ? w[5] : w[4]);
-    if (nref & FP_REF_LEAF) {
-        L.active = false;
-        int32_t leaf_id = -1;
-        if (MODE == FP_MODE_LEAVES) leaf_id = p.deep_leaf[4 * (int64_t)L.ref + 2 * d0 + d1];
-        finish<MODE>(p, svotes, row0, L.r, L.t, nref & 0x7FFFFFFFu, leaf_id);
-    } else if (nref > L.ref && (int64_t)nref < p.n_super) {  // forward only, so every walk ends
-        L.ref = nref;
-    } else {
-        report(p.status, FP_ERR_FLAG_DEVICE);
-        L.active = false;
-    }
+    // forward only, so every walk ends: 1 <= next - ref <= n_super - 1 - ref
+    const bool ahead = s.next - ref - 1u < p.n_super - 1u - ref;
+    const bool go = on && !s.leaf;
+    if (go && !ahead) L.bad = 1;
+    L.ref = go && ahead ? s.next : FP_NO_TASK;
 }
 
-// CTA-wide state shared by the items a CTA runs.
-struct CtaShared {
-    uint64_t full[FP_NBUF];   // block staged (bulk copy done)
-    int task_next[FP_NBUF];   // next unclaimed task of the buffer's bin
-    int claim_done[FP_NBUF];  // warps done claiming the buffer's bin
-    int issued[FP_NBUF];      // bulk copies issued into the buffer
-    int use0[FP_NBUF];        // issued[] when the current item started
-    int last;
-    int abort;
-    long long next_item;
-};
+// The walk of one row (at xb) through the head of tree column k of the bin
+// block at offset blk, whose exits begin at `exits`: the offset of the exit
+// word it ends on, or FP_NO_EXIT (corrupt ranked heads only).  HK: the head
+// kind when known at compile time (0 ranked, 1 level slots, 2 paired level
+// slots), or -1 to read it from p.levels (the batched kernel, whose forests
+// may differ).  Record q of a level head lies at at0 + q * rec and exit e
+// where record nranks + e would, scaled to 4-byte words, so the walks keep
+// the record's offset itself and never its index.
+#define FP_NO_EXIT 0xFFFFFFFFu
+
+template <bool KEYS, int HK>
+__device__ __forceinline__ uint32_t head_walk(const TravParams &p, const uint8_t *smem, uint32_t blk, uint32_t exits,
+                                              int k, int stride, int nranks, int nexits, uint32_t xb, bool my) {
+    const int levels = HK >= 0 ? HK : p.levels;
+    if (levels == 2) {
+        // paired slots: a node and its two children per 16-byte record,
+        // successors 4q+1 .. 4q+4; (depth+1)/2 records per walk
+        const uint32_t rec = (uint32_t)stride * 16u, at0 = blk + (uint32_t)k * 16u;
+        const uint32_t left = rec - 3u * at0, right = left + 2u * rec;
+        uint32_t at = at0;
+#pragma unroll 1  // measured: unrolling the head walk only adds instructions
+        for (int l = 0; l <= p.depth; l += 2) {
+            const uint4 nd = lds128(smem, at);
+            const bool r0 = !goes_left<KEYS>(lds(smem, xb + ((nd.w & 1023u) << 7)), nd.x);
+            const uint32_t f1 = nd.w >> (r0 ? 20 - 7 : 10 - 7);
+            const bool r1 = !goes_left<KEYS>(lds(smem, xb + (f1 & (1023u << 7))), r0 ? nd.z : nd.y);
+            at = 4u * at + (r0 ? right : left) + (r1 ? rec : 0u);
+        }
+        return exits + ((at - exits) >> 2);
+    }
+    if (levels) {
+        // implicit slots: every walk takes depth+1 steps, children 2s+1, 2s+2
+        const uint32_t rec = (uint32_t)stride * 8u, at0 = blk + (uint32_t)k * 8u;
+        const uint32_t left = rec - at0, right = left + rec;
+        uint32_t at = at0;
+#pragma unroll 1
+        for (int l = 0; l <= p.depth; ++l) {
+            const uint2 nd = *reinterpret_cast<const uint2 *>(smem + at);
+            at = 2u * at + (goes_left<KEYS>(lds(smem, xb + ((nd.y >> 22) << 7)), nd.x) ? left : right);
+        }
+        return exits + ((at - exits) >> 1);
+    }
+    const uint2 *hn = reinterpret_cast<const uint2 *>(smem + blk) + k;  // this tree's column of the block
+    uint32_t hr = 0;  // head rank, then nranks + exit index
+    bool busy = my;
+    while (__any_sync(0xffffffffu, busy)) {  // ranked heads: until the last lane leaves
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {  // two steps per vote
+            if (busy) {
+                const uint2 nd = hn[hr * stride];
+                const uint32_t m = nd.y;
+                uint32_t nh = goes_left<KEYS>(lds(smem, xb + ((m >> 22) << 7)), nd.x)
+                                  ? (m & FP_TARGET_MASK)
+                                  : ((m >> FP_TARGET_BITS) & FP_TARGET_MASK);
+                busy = nh < (uint32_t)nranks;
+                if (busy && nh <= hr) {  // ranks grow along every path of a valid block
+                    busy = false;
+                    nh = (uint32_t)(nranks + nexits);
+                }
+                hr = nh;
+            }
+        }
+    }
+    const uint32_t e = hr - (uint32_t)nranks;
+    return e < (uint32_t)nexits ? exits + 4u * (e * (uint32_t)stride + (uint32_t)k) : FP_NO_EXIT;
+}
+
+// Forests whose trees end in the interleaved heads (no super-nodes: shallow
+// trees, such as boosted ones).  Every walk of a slab through a tree ends
+// together, so nothing is pushed or popped: a warp takes a slab and a run of
+// up to 8 of the bin's trees, keeps the row's sum of leaf values (or its votes
+// for class 1 of 2) in a register over the run, and adds it to the slab's
+// counter once.  A task costs the head walk, one exit word and one add; as a
+// burst of its own it also paid for the claim, its division, the read of its
+// value from global memory and an atomic (256 boosted trees of six levels, 2 M
+// rows: 2.93 ms as bursts, 1.53 ms as runs; bound by instruction issue).
+template <int MODE, bool KEYS, int HK>
+__device__ __forceinline__ void walk_heads(const TravParams &p, uint8_t *smem, CtaShared &sh, const FpBin &bn,
+                                           uint32_t blk, uint32_t exits, int buf, int rows, int G, uint32_t inv_g,
+                                           int &bad) {
+    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    // runs of 8 trees, shorter when the bin would leave warps without one
+    const int run = max(1, min(8, bn.width * G / nwarps));
+    const int units = (bn.width + run - 1) / run * G;
+    for (;;) {
+        int unit = 0;
+        if (lane == 0) unit = atomicAdd(&sh.next[buf], 1);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        if (unit >= units) break;
+        const int c = G > 1 ? (int)__umulhi((uint32_t)unit, inv_g) : unit, g = unit - c * G;
+        const uint32_t xb = (uint32_t)g * p.slab + (uint32_t)lane * 4u;
+        const int r = g * 32 + lane;
+        const bool my = r < rows;
+        const int k1 = min(bn.width, (c + 1) * run);
+        float sum = 0.0f;
+        uint32_t ones = 0;
+        for (int k = c * run; k < k1; ++k) {
+            const uint32_t at = head_walk<KEYS, HK>(p, smem, blk, exits, k, bn.stride, bn.nranks, bn.nexits, xb, my);
+            if (HK <= 0 && at == FP_NO_EXIT) {
+                bad |= my;
+                continue;
+            }
+            if (MODE == FP_MODE_VALUES) {
+                sum += __uint_as_float(lds(smem, at));  // the exits hold the leaves' values themselves
+            } else if (MODE == FP_MODE_LEAVES) {
+                if (my)
+                    put_leaf(p, sh, (uint32_t)r | ((uint32_t)(bn.first_tree + k) << 11),
+                             p.pheads[(bn.phead_off >> 2) + ((at - exits) >> 2)]);
+            } else {
+                const uint32_t cls = lds(smem, at) & 0x7FFFFFFFu;
+                if (p.C == 2) {
+                    ones += cls & 1u;
+                    bad |= my && cls > 1u;
+                } else {
+                    bad |= !vote(p, smem, my, xb, cls);
+                }
+            }
+        }
+        if (MODE == FP_MODE_VALUES && my) add_value(p, smem, xb, sum);
+        if (MODE == FP_MODE_VOTES && my && p.C == 2 && ones)
+            atomicAdd(reinterpret_cast<uint32_t *>(smem + xb + (((uint32_t)p.F + 1u) << 7)), ones);
+    }
+}
 
 __device__ __forceinline__ void cta_init(CtaShared &sh) {
     if (threadIdx.x == 0) {
@@ -420,34 +603,31 @@ __device__ __forceinline__ void cta_finish(CtaShared &sh) {
 // goes through buffer bi % nbuf; the k-th copy ever issued into a buffer
 // completes its barrier's phase k, so a wait needs the buffer's copy count
 // at the item's start (use0) plus bi / nbuf.  Counting per buffer keeps the
-// phases right when items of forests with different nbuf share a CTA.
-// HK: the head kind when known at compile time (0 ranked, 1 level slots,
-// 2 paired level slots), or -1 to read it from p.levels (the batched kernel,
-// whose forests may differ).
-template <int MODE, int DK, int HK>
+// phases right when items of forests with different nbuf share a CTA.  Every
+// warp waits for every bin's block, also for one it has no unit in: a warp
+// that ran ahead of a buffer's phases could not tell them apart.
+// HEADS: the forest has no super-nodes (walk_heads); its own build, since the
+// two walks in one kernel cost the other 8 % more instructions.
+template <int MODE, int DK, int HK, bool HEADS>
 __device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint8_t *smem, CtaShared &sh) {
     constexpr bool D3 = DK >= 3;  // rows and thresholds are (remapped) order keys
     constexpr bool LEAVES = MODE == FP_MODE_LEAVES, VALUES = MODE == FP_MODE_VALUES;
     const int levels = HK >= 0 ? HK : p.levels;
     const int R = p.R, F = p.F, C = p.C;
-    uint32_t *xs = reinterpret_cast<uint32_t *>(smem);  // the tile's rows: (remapped) order keys or float bits
-    const int xs_bytes = ((F * R * 4) + 15) & ~15;
+    const int VR = LEAVES ? 0 : (VALUES ? 1 : C);  // counters per row: class votes, or one float sum
+    const uint32_t slab = p.slab;
+    const uint32_t hbuf0 = (uint32_t)(R >> 5) * slab;  // nbuf bin-block buffers, head_smem bytes each
     const int nbuf = p.nbuf;
-    uint8_t *const hbuf0 = smem + xs_bytes;  // nbuf bin-block buffers, head_smem bytes each
-    uint32_t *svotes = reinterpret_cast<uint32_t *>(smem + xs_bytes + nbuf * p.head_smem);
-    const int CS = VALUES ? 1 : C;  // counters per row: class votes, or one float sum
-    const int vote_bytes = LEAVES ? 0 : ((R * CS * 4) + 15) & ~15;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    uint2 *ring = reinterpret_cast<uint2 *>(smem + xs_bytes + nbuf * p.head_smem + vote_bytes) + warp * FP_RING;
+    uint2 *ring = reinterpret_cast<uint2 *>(smem + hbuf0 + (uint32_t)(nbuf * p.head_smem)) + warp * FP_RING;
     const unsigned lt_mask = (1u << lane) - 1u;
 
-    // one thread: stage bin b of the pass, the item's bi-th bin
-    auto issue = [&](int b, int bi) {
-        const int buf = bi % nbuf;
-        sh.task_next[buf] = 0;
-        sh.claim_done[buf] = 0;
+    // one thread: stage bin b into a buffer
+    auto issue = [&](int b, int buf) {
+        sh.next[buf] = 0;
+        sh.done[buf] = 0;
         sh.issued[buf] += 1;
-        stage_block_bulk(p, b, hbuf0 + buf * p.head_smem, &sh.full[buf]);
+        stage_block_bulk(p, b, smem + hbuf0 + buf * p.head_smem, &sh.full[buf]);
     };
 
     // A CTA that gave up a wait skips its remaining items; each one records
@@ -462,94 +642,84 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint
     const int64_t tile = item - (int64_t)pass * p.n_tiles;
     const int64_t row0 = tile * R;
     const int rows = (int)(p.n - row0 < (int64_t)R ? p.n - row0 : (int64_t)R);
-    const FpPass ps = p.passes[pass];
-    const int nbins = ps.bin_end - ps.bin_begin;
-    const float inv_rows = 1.0f / (float)rows;
+    const int G = (rows + 31) >> 5;  // slabs in use
 
-    // 1. rows (feature-major, as order keys) -> shared memory; 2. the first
-    //    bins' blocks in flight
-    const float *src = p.X + row0 * F;
-    const bool vec_rows = (F & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
-    {
-        if (vec_rows) {
-            // lane = row: 16-byte loads along the row, and each store of a
-            // warp writes 32 consecutive rows of one feature (32 banks).  The
-            // work is cut into units of 32 rows x 16 features, dealt out to
-            // all warps, so that a tile of few wide rows (784 features, 64
-            // rows) is staged by every warp, not by two
-            const int nq = F >> 2;
-            const int groups = (rows + 31) >> 5, qblocks = (nq + 3) >> 2;
-            for (int u = warp; u < groups * qblocks; u += nwarps) {
-                const int g = u % groups, q0 = (u / groups) * 4;
-                const int r = g * 32 + lane;
-                if (r < rows) {
-                    const float4 *rp = reinterpret_cast<const float4 *>(src + (int64_t)r * F);
-                    uint32_t *dst = xs + r;
-                    if (q0 + 4 <= nq) {
-                        float4 v[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) v[k] = __ldg(rp + q0 + k);
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            uint32_t *d = dst + (4 * (q0 + k)) * R;
-                            d[0] = staged<DK>(p, v[k].x);
-                            d[R] = staged<DK>(p, v[k].y);
-                            d[2 * R] = staged<DK>(p, v[k].z);
-                            d[3 * R] = staged<DK>(p, v[k].w);
-                        }
-                    } else {
-                        for (int q = q0; q < nq; ++q) {
-                            const float4 v = __ldg(rp + q);
-                            uint32_t *d = dst + (4 * q) * R;
-                            d[0] = staged<DK>(p, v.x);
-                            d[R] = staged<DK>(p, v.y);
-                            d[2 * R] = staged<DK>(p, v.z);
-                            d[3 * R] = staged<DK>(p, v.w);
-                        }
-                    }
-                }
-            }
-        } else {
-            const int total = rows * F;
-            for (int e = tid; e < total; e += blockDim.x) {
-                const int r = e / F;
-                cp_async4(xs + (e - r * F) * R + r, src + e);
-            }
-        }
-        cp_async_commit();
-    }
+    // 1. rows -> shared memory, as order keys; 2. the first bins' blocks in flight
     if (tid == 0) {
-        for (int i = 0; i < FP_NBUF; ++i) sh.use0[i] = sh.issued[i];
-        if (!sh.abort)
-            for (int i = 0; i < nbuf && i < nbins; ++i) issue(ps.bin_begin + i, i);
-
+        const FpPass ps = p.passes[pass];
+        sh.bin0 = ps.bin_begin;
+        sh.bin1 = ps.bin_end;
+        sh.tile = tile;
+        uint32_t ph = 0;
+        for (int i = 0; i < FP_NBUF; ++i) ph |= ((uint32_t)sh.issued[i] & 1u) << i;
+        sh.phases = ph;
+        for (int i = 0; i < nbuf && ps.bin_begin + i < ps.bin_end; ++i) issue(ps.bin_begin + i, i);
     }
-    if (!LEAVES)
-        for (int i = tid; i < R * CS; i += blockDim.x) svotes[i] = 0;
-    cp_async_wait_all();
-    if (D3 && !vec_rows) {  // each thread turns the values it copied into keys
-        const int total = rows * F;
-        for (int e = tid; e < total; e += blockDim.x) {
-            const int r = e / F;
-            uint32_t *x = xs + (e - r * F) * R + r;
-            *x = staged<DK>(p, __uint_as_float(*x));
+    {
+        // lane = row of a slab, 16 features at a time: loads along the row,
+        // and each store of a warp fills the 32 columns of one feature.  The
+        // (slab, 16 features) units are dealt out to all warps, so that a
+        // tile of few wide rows (784 features, 64 rows) is staged by every
+        // warp, not by two.
+        const float *src = p.X + row0 * F;
+        const bool vec_rows = (F & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
+        const int fblocks = (F + 15) >> 4;
+        for (int u = warp; u < G * fblocks; u += nwarps) {
+            const int fq = u / G, g = u - fq * G, f0 = fq * 16;
+            const int r = g * 32 + lane;
+            if (r >= rows) continue;
+            const float *rp = src + (int64_t)r * F + f0;
+            uint32_t *dst = reinterpret_cast<uint32_t *>(smem + (uint32_t)g * slab) + f0 * 32 + lane;
+            auto put4 = [&](int k, float4 v) {
+                uint32_t *d = dst + 128 * k;
+                d[0] = staged<DK>(p, v.x);
+                d[32] = staged<DK>(p, v.y);
+                d[64] = staged<DK>(p, v.z);
+                d[96] = staged<DK>(p, v.w);
+            };
+            const float4 *rq = reinterpret_cast<const float4 *>(rp);
+            if (vec_rows && f0 + 16 <= F) {
+                float4 v[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) v[k] = __ldg(rq + k);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) put4(k, v[k]);
+            } else if (vec_rows) {
+                for (int k = 0; f0 + 4 * k < F; ++k) put4(k, __ldg(rq + k));
+            } else {
+                const int m = F - f0 < 16 ? F - f0 : 16;
+#pragma unroll 4
+                for (int k = 0; k < m; ++k) dst[32 * k] = staged<DK>(p, __ldg(rp + k));
+            }
         }
+    }
+    for (int u = warp; u < G * VR; u += nwarps) {
+        const int g = u / VR;
+        reinterpret_cast<uint32_t *>(smem + (uint32_t)g * slab)[(F + u - g * VR) * 32 + lane] = 0;
     }
     __syncthreads();
 
     LaneTask L;
-    L.active = false;
-    L.r = 0;
-    L.t = 0;
-    L.ref = 0;
+    L.ref = FP_NO_TASK;
+    L.xb = 0;
+    L.rt = 0;
+    L.bad = 0;
+    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    Pending pend;
+    pend.on = false;
+    pend.at = 0;
+    pend.word = 0;
     int head = 0, tail = 0;  // warp-uniform ring cursors
 
-    const int u0 = sh.use0[0], u1 = sh.use0[1], u2 = sh.use0[2];  // read after the barrier above
-    for (int bi = 0; bi < nbins; ++bi) {
-        const int buf = bi % nbuf;
+    // unit u of a bin is slab u % G of its tree u / G: ceil(2^32 / G) divides by G
+    const uint32_t inv_g = G > 1 ? 0xFFFFFFFFu / (uint32_t)G + 1u : 0u;
+
+    uint32_t phases = sh.phases;  // bit b: the phase parity that buffer b's next block completes
+    int buf = 0;
+    for (int b = sh.bin0; b < sh.bin1; ++b) {
         {  // wait until the bin's block has landed
-            const int ub = buf == 0 ? u0 : (buf == 1 ? u1 : u2);
-            const uint32_t parity = (uint32_t)(ub + bi / nbuf) & 1u;
+            const uint32_t parity = (phases >> buf) & 1u;
+            phases ^= 1u << buf;
             bool ok = false;
             for (int spin = 0; spin < p.spin_limit; ++spin) {
                 if (*(volatile int *)&sh.abort) break;
@@ -566,210 +736,186 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint
                 break;
             }
         }
-        const int b = ps.bin_begin + bi;
         const FpBin bn = p.bins[b];
         const int stride = bn.stride, nranks = bn.nranks, nexits = bn.nexits;
-        const int ntask = rows * bn.width;
-        const uint8_t *blk = hbuf0 + buf * p.head_smem;
-        const uint2 *hnode = reinterpret_cast<const uint2 *>(blk);
-        const uint32_t *hexit =
-            reinterpret_cast<const uint32_t *>(blk + (size_t)nranks * stride * (levels == 2 ? 16 : 8));
+        const uint32_t blk = hbuf0 + (uint32_t)(buf * p.head_smem);
+        const uint32_t exits = blk + (uint32_t)(nranks * stride * (levels == 2 ? 16 : 8));
 
-        for (;;) {
-            uint32_t w[8];
-            if (L.active) deep_issue(p, L, w);  // in flight during the burst below
+        if (HEADS) walk_heads<MODE, D3, HK>(p, smem, sh, bn, blk, exits, buf, rows, G, inv_g, L.bad);
+        const int units = bn.width * G;
+        while (!HEADS) {
+            ld_super(p.deep, L.ref, w);  // in flight during the burst below
+            settle<MODE>(p, smem, sh, pend);
             if (tail - head <= p.refill) {
-                // burst: 32 consecutive tasks through the head, all lanes together
-                int base = 0;
-                if (lane == 0) base = atomicAdd(&sh.task_next[buf], 32);
-                base = __shfl_sync(0xffffffffu, base, 0);
-                if (base >= ntask) {  // the bin is claimed out: use the load in flight, then move on
-                    if (L.active) deep_finish<MODE, DK>(p, xs, svotes, row0, L, w);
-                    pop_tasks(p, ring, head, tail, L, lt_mask);
+                // burst: the unit's 32 rows through the head of its tree, all lanes together
+                int unit = 0;
+                if (lane == 0) unit = atomicAdd(&sh.next[buf], 1);
+                unit = __shfl_sync(0xffffffffu, unit, 0);
+                if (unit >= units) {  // all taken: use the load in flight, then move on
+                    if (__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) deep_finish<MODE, DK>(p, smem, L, pend, w);
+                    pop_tasks<MODE>(p, ring, head, tail, L, lt_mask);
                     break;
                 }
-                const bool my = lane < ntask - base;
-                const int task = base + lane;
-                // task / rows by a float reciprocal, corrected to the exact quotient
-                int k2 = my ? (int)((float)task * inv_rows) : 0;
-                if (my) {
-                    k2 -= k2 * rows > task;
-                    k2 += (k2 + 1) * rows <= task;
-                }
-                const int r2 = my ? task - k2 * rows : 0;
-                uint32_t hr = 0;  // head rank (or slot), then nranks + exit index
-                const uint2 *hn = hnode + k2;  // this lane's tree column of the block
-                const uint32_t *xr = xs + r2;  // this lane's row
-                if (levels == 2) {
-                    // paired slots: a node and its two children per 16-byte record,
-                    // successors 4q+1 .. 4q+4; (depth+1)/2 records per walk
-                    const uint4 *hq = reinterpret_cast<const uint4 *>(blk) + k2;
-#pragma unroll 1  // measured: unrolling the head walk only adds instructions
-                    for (int l = 0; l <= p.depth; l += 2) {
-                        const uint4 nd = hq[hr * stride];
-                        const uint32_t x0 = xr[(nd.w & 1023u) * R];
-                        const uint32_t d0 = goes_left<D3>(x0, nd.x) ? 0u : 1u;
-                        const uint32_t f1 = d0 ? (nd.w >> 20) & 1023u : (nd.w >> 10) & 1023u;
-                        const uint32_t x1 = xr[f1 * R];
-                        const uint32_t d1 = goes_left<D3>(x1, d0 ? nd.z : nd.y) ? 0u : 1u;
-                        hr = 4 * hr + 1 + 2 * d0 + d1;
-                    }
-                } else if (levels) {
-                    // implicit slots: every walk takes depth+1 steps, children 2s+1, 2s+2
-#pragma unroll 1
-                    for (int l = 0; l <= p.depth; ++l) {
-                        const uint2 nd = hn[hr * stride];
-                        const uint32_t xv = xr[(nd.y >> 22) * R];
-                        hr = 2 * hr + (goes_left<D3>(xv, nd.x) ? 1u : 2u);
-                    }
-                }
-                bool busy = my && !levels;
-                while ((HK <= 0 || levels == 0) && __any_sync(0xffffffffu, busy)) {  // ranked heads only
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {  // two steps per vote
-                        if (busy) {
-                            const uint2 nd = hn[hr * stride];
-                            const uint32_t m = nd.y;
-                            uint32_t nh = goes_left<D3>(xr[(m >> 22) * R], nd.x)
-                                              ? (m & FP_TARGET_MASK)
-                                              : ((m >> FP_TARGET_BITS) & FP_TARGET_MASK);
-                            busy = nh < (uint32_t)nranks;
-                            if (busy && nh <= hr) {  // ranks grow along every path of a valid block
-                                report(p.status, FP_ERR_FLAG_DEVICE);
-                                busy = false;
-                                nh = (uint32_t)(nranks + nexits);
-                            }
-                            hr = nh;
-                        }
-                    }
-                }
-                const uint32_t e = hr - (uint32_t)nranks;
-                const uint32_t er = (my && e < (uint32_t)nexits) ? hexit[e * stride + k2] : FP_NO_CLASS;
-                const int t2 = bn.first_tree + k2;
-                if (my && (er & FP_REF_LEAF)) {
-                    int32_t leaf_id = -1;
-                    if (LEAVES && e < (uint32_t)nexits) leaf_id = p.pheads[(bn.phead_off >> 2) + e * stride + k2];
-                    finish<MODE>(p, svotes, row0, r2, t2, er & 0x7FFFFFFFu, leaf_id);
-                }
+                const int uk = G > 1 ? (int)__umulhi((uint32_t)unit, inv_g) : unit, ug = unit - uk * G;
+                const uint32_t xb = (uint32_t)ug * slab + (uint32_t)lane * 4u;
+                const int r2 = ug * 32 + lane;
+                const bool my = r2 < rows;
+                const uint32_t at =
+                    head_walk<D3, HK>(p, smem, blk, exits, uk, stride, nranks, nexits, xb, my);
+                const bool ok = HK > 0 || at != FP_NO_EXIT;
+                const uint32_t er = ok ? lds(smem, at) : FP_NO_CLASS;
                 const bool push = my && !(er & FP_REF_LEAF);
+                if (my && !push) {  // a leaf in the head, or right below it
+                    const uint32_t cls = er & 0x7FFFFFFFu;
+                    if (LEAVES) {
+                        L.bad |= !ok;
+                        if (ok)
+                            put_leaf(p, sh, (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11),
+                                     p.pheads[(bn.phead_off >> 2) + ((at - exits) >> 2)]);
+                    } else if (VALUES) {
+                        L.bad |= cls >= p.n_vals;
+                        if (cls < p.n_vals) add_value(p, smem, xb, __ldg(p.leaf_val + cls));
+                    } else {
+                        L.bad |= !vote(p, smem, true, xb, cls);
+                    }
+                }
                 const unsigned pm = __ballot_sync(0xffffffffu, push);
                 if (push)
                     ring[(tail + __popc(pm & lt_mask)) & (FP_RING - 1)] =
-                        make_uint2(er, (uint32_t)r2 | ((uint32_t)t2 << 11));
+                        make_uint2(er, LEAVES ? (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11) : xb);
                 tail += __popc(pm);
                 __syncwarp();
             }
-            if (L.active) deep_finish<MODE, DK>(p, xs, svotes, row0, L, w);
-            pop_tasks(p, ring, head, tail, L, lt_mask);
+            if (__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) deep_finish<MODE, DK>(p, smem, L, pend, w);
+            pop_tasks<MODE>(p, ring, head, tail, L, lt_mask);
         }
         // this warp reads the bin's block no more; the last warp refills the buffer
         __syncwarp();
         if (lane == 0) {
-            const int done = atomicAdd(&sh.claim_done[buf], 1);
-            if (done == nwarps - 1 && bi + nbuf < nbins && !*(volatile int *)&sh.abort)
-                issue(ps.bin_begin + bi + nbuf, bi + nbuf);
+            const int done = atomicAdd(&sh.done[buf], 1);
+            if (done == nwarps - 1 && b + nbuf < sh.bin1 && !*(volatile int *)&sh.abort) issue(b + nbuf, buf);
         }
+        if (++buf == nbuf) buf = 0;
         __syncwarp();
     }
     const bool aborted = *(volatile int *)&sh.abort != 0;
     // drain: the item's last pending and running tasks
-    for (; !aborted;) {
+    for (; !HEADS && !aborted;) {
         __syncwarp();
-        pop_tasks(p, ring, head, tail, L, lt_mask);
-        if (!__any_sync(0xffffffffu, L.active)) break;
-        if (L.active) {
-            uint32_t w[8];
-            deep_issue(p, L, w);
-            deep_finish<MODE, DK>(p, xs, svotes, row0, L, w);
-        }
+        pop_tasks<MODE>(p, ring, head, tail, L, lt_mask);
+        if (!__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) break;
+        ld_super(p.deep, L.ref, w);
+        settle<MODE>(p, smem, sh, pend);
+        deep_finish<MODE, DK>(p, smem, L, pend, w);
     }
+    settle<MODE>(p, smem, sh, pend);
+    if (L.bad) report(p.status, FP_ERR_FLAG_DEVICE);
     __syncthreads();
+
+    // what the walk did not keep in registers
+    const int64_t base = sh.tile * p.R;
+    const int nrows = (int)(p.n - base < (int64_t)p.R ? p.n - base : (int64_t)p.R);
 
     // 5. values: bias + scale * the row's sum (several passes: summed in global
     //    memory, the CTA finishing a tile's last pass writes the result)
     if (VALUES && !*(volatile int *)&sh.abort) {
-        const float *sv = reinterpret_cast<const float *>(svotes);
+        auto sum_of = [&](int rr) {
+            return __uint_as_float(lds(smem, (uint32_t)(rr >> 5) * slab + ((uint32_t)F << 7) + (uint32_t)(rr & 31) * 4u));
+        };
         if (p.n_passes == 1) {
-            for (int rr = tid; rr < rows; rr += blockDim.x) p.out_val[row0 + rr] = p.vbias + p.vscale * sv[rr];
+            for (int rr = tid; rr < nrows; rr += blockDim.x) p.out_val[base + rr] = p.vbias + p.vscale * sum_of(rr);
         } else {
-            float *dst = p.acc_val + row0;
-            for (int rr = tid; rr < rows; rr += blockDim.x) {
-                const float v = sv[rr];
+            float *dst = p.acc_val + base;
+            for (int rr = tid; rr < nrows; rr += blockDim.x) {
+                const float v = sum_of(rr);
                 if (v != 0.0f) atomicAdd(dst + rr, v);
             }
             __threadfence();
             __syncthreads();
-            if (tid == 0) sh.last = atomicAdd(p.tile_done + tile, 1u) == (unsigned)(p.n_passes - 1);
+            if (tid == 0) sh.last = atomicAdd(p.tile_done + sh.tile, 1u) == (unsigned)(p.n_passes - 1);
             __syncthreads();
             if (sh.last) {
                 __threadfence();
-                for (int rr = tid; rr < rows; rr += blockDim.x)
-                    p.out_val[row0 + rr] = p.vbias + p.vscale * __ldcg(dst + rr);
+                for (int rr = tid; rr < nrows; rr += blockDim.x)
+                    p.out_val[base + rr] = p.vbias + p.vscale * __ldcg(dst + rr);
             }
         }
     }
-    // 5. votes and class
+    // 5. votes and class: a thread per row; class 0 has the votes that no other class got
     if (MODE == FP_MODE_VOTES && !*(volatile int *)&sh.abort) {
-        if (p.n_passes == 1) {
-            if (p.out_votes) {  // counters are class-major (svotes[c * R + r]), the output row-major
-                uint32_t *dst = p.out_votes + row0 * C;
-                for (int i = tid; i < rows * C; i += blockDim.x) {
-                    const int rr = i / C;
-                    dst[i] = svotes[(i - rr * C) * R + rr];
+        const FpBin first = p.bins[sh.bin0], last = p.bins[sh.bin1 - 1];
+        const uint32_t trees = (uint32_t)(last.first_tree + last.width - first.first_tree);
+        uint32_t *const dst = p.n_passes == 1 ? p.out_votes : p.acc;
+        for (int rr = tid; rr < nrows; rr += blockDim.x) {
+            const uint32_t vb = (uint32_t)(rr >> 5) * slab + ((uint32_t)F << 7) + (uint32_t)(rr & 31) * 4u;
+            uint32_t *d = dst ? dst + (base + rr) * C : nullptr;
+            uint32_t rest = trees, bv = 0;
+            int best = 0;
+            for (int c = 1; c < C; ++c) {
+                const uint32_t v = lds(smem, vb + (uint32_t)c * 128u);
+                rest -= v;
+                if (v > bv) { bv = v; best = c; }
+                if (p.n_passes == 1) {
+                    if (d) d[c] = v;
+                } else if (v) {
+                    atomicAdd(d + c, v);
                 }
             }
-            if (p.out_class) {
-                for (int rr = tid; rr < rows; rr += blockDim.x) {
-                    const uint32_t *v = svotes + rr;
-                    int best = 0;
-                    uint32_t bv = v[0];
-                    for (int c = 1; c < C; ++c)
-                        if (v[c * R] > bv) { bv = v[c * R]; best = c; }
-                    p.out_class[row0 + rr] = best;
-                }
+            if (p.n_passes == 1) {
+                if (d) d[0] = rest;
+                if (p.out_class) p.out_class[base + rr] = rest >= bv ? 0 : best;
+            } else if (rest) {
+                atomicAdd(d, rest);
             }
-        } else {
-            uint32_t *dst = p.acc + row0 * C;
-            for (int i = tid; i < rows * C; i += blockDim.x) {
-                const int rr = i / C;
-                const uint32_t v = svotes[(i - rr * C) * R + rr];
-                if (v) atomicAdd(dst + i, v);
-            }
-            if (p.out_class) {
+        }
+        if (p.n_passes > 1 && p.out_class) {
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) sh.last = atomicAdd(p.tile_done + sh.tile, 1u) == (unsigned)(p.n_passes - 1);
+            __syncthreads();
+            if (sh.last) {
                 __threadfence();
-                __syncthreads();
-                if (tid == 0) sh.last = atomicAdd(p.tile_done + tile, 1u) == (unsigned)(p.n_passes - 1);
-                __syncthreads();
-                if (sh.last) {
-                    __threadfence();
-                    for (int rr = tid; rr < rows; rr += blockDim.x) {
-                        const uint32_t *v = dst + rr * C;
-                        int best = 0;
-                        uint32_t bv = __ldcg(v);
-                        for (int c = 1; c < C; ++c) {
-                            const uint32_t w = __ldcg(v + c);
-                            if (w > bv) { bv = w; best = c; }
-                        }
-                        p.out_class[row0 + rr] = best;
+                for (int rr = tid; rr < nrows; rr += blockDim.x) {
+                    const uint32_t *v = p.acc + (base + rr) * C;
+                    int best = 0;
+                    uint32_t bv = __ldcg(v);
+                    for (int c = 1; c < C; ++c) {
+                        const uint32_t x = __ldcg(v + c);
+                        if (x > bv) { bv = x; best = c; }
                     }
+                    p.out_class[base + rr] = best;
                 }
             }
         }
     }
     __syncthreads();  // the next item reuses shared memory
+}
 
+// Forests with leaf values and no super-nodes: every exit of the heads becomes
+// the value of the leaf that it names (once, after the upload), so that a
+// walk ends on the value instead of on its slot in a table in global memory.
+// One block per bin.
+__global__ void fp_inline_values_kernel(uint8_t *heads, const FpBin *bins, const float *leaf_val, uint32_t n_vals,
+                                        uint32_t node_bytes) {
+    const FpBin bn = bins[blockIdx.x];
+    uint32_t *exits = reinterpret_cast<uint32_t *>(heads + bn.head_off + (size_t)bn.nranks * bn.stride * node_bytes);
+    for (int i = threadIdx.x; i < bn.nexits * bn.stride; i += blockDim.x) {
+        const uint32_t slot = exits[i] & 0x7FFFFFFFu;
+        exits[i] = slot < n_vals ? __float_as_uint(leaf_val[slot]) : 0u;  // entries that no walk reaches: 0
+    }
 }
 
 // MINB = 1: one CTA of up to 1024 threads per SM (up to 64 registers a thread);
 // MINB = 2: CTAs of up to 768 threads, at most 42 registers a thread, so that
 // two 24-warp or three 16-warp CTAs share an SM when shared memory allows:
 // more warps to hide the latency of the dependent loads of each walk.
-template <int MODE, int MINB, int DK, int HK>
+template <int MODE, int MINB, int DK, int HK, bool HEADS>
 __global__ void __launch_bounds__(MINB == 1 ? 1024 : 768, MINB) fp_traverse_kernel(const TravParams p) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ CtaShared sh;
     cta_init(sh);
-    for (int64_t item = blockIdx.x; item < p.n_items; item += gridDim.x) run_item<MODE, DK, HK>(p, item, smem, sh);
+    for (int64_t item = blockIdx.x; item < p.n_items; item += gridDim.x) 
+        run_item<MODE, DK, HK, HEADS>(p, item, smem, sh);
     cta_finish(sh);
 }
 
@@ -803,11 +949,11 @@ __global__ void __launch_bounds__(1024, 1) fp_traverse_batched_kernel(const __gr
         int j = 0;
         while (j + 1 < bp.k && bp.item_begin[j + 1] <= item) ++j;
         if (KIND == 3 || (KIND == 0 && bp.p[j].deep_kind == 3))
-            run_item<FP_MODE_VOTES, 3, HK>(bp.p[j], item - bp.item_begin[j], smem, sh);
+            run_item<FP_MODE_VOTES, 3, HK, false>(bp.p[j], item - bp.item_begin[j], smem, sh);
         else if (KIND == 4 || (KIND == 0 && bp.p[j].deep_kind == 4))
-            run_item<FP_MODE_VOTES, 4, HK>(bp.p[j], item - bp.item_begin[j], smem, sh);
+            run_item<FP_MODE_VOTES, 4, HK, false>(bp.p[j], item - bp.item_begin[j], smem, sh);
         else
-            run_item<FP_MODE_VOTES, 2, HK>(bp.p[j], item - bp.item_begin[j], smem, sh);
+            run_item<FP_MODE_VOTES, 2, HK, false>(bp.p[j], item - bp.item_begin[j], smem, sh);
     }
     cta_finish(sh);
 }
