@@ -109,10 +109,15 @@ typedef struct fp_forest_desc {
  *                     wide rows ~200 KiB; shrunk at upload to fit shared
  *                     memory)
  *   warps_per_cta     warps per CTA of the traversal kernel, 1..32
- *   pass_bytes        bins are swept in groups ("passes") whose records fit in
- *                     this many bytes, so a pass stays resident in L2 while
- *                     every observation tile walks it; 0 = default (48 MiB),
- *                     negative = one pass over the whole forest
+ *   pass_bytes        bins are grouped into "passes" whose records fit in this
+ *                     many bytes; 0 = default (48 MiB), negative = one pass
+ *                     over the whole forest.  A forest of several passes that
+ *                     is larger than L2, with tiles too small to share its
+ *                     lines, is swept pass by pass, so that a pass stays
+ *                     resident in L2 while every observation tile walks it;
+ *                     else large batches sweep all passes at once, and small
+ *                     ones split the forest's bins over the GPU in a way that
+ *                     needs scratch (fp_predict_noalloc)
  *   refill_lanes      a warp hands new (observation, tree) tasks to its idle
  *                     lanes once this many lanes are idle, 1..32
  *   head_select       which 2^(d+1)-1 nodes of a tree form its interleaved head:
@@ -220,8 +225,11 @@ int fp_configure(fp_device_forest *forest, const fp_pack_params *params);
  *   out_class  device, [n] int32 argmax of the votes (lowest class on ties),
  *              or NULL
  * Asynchronous on `stream`; X must stay valid and the outputs untouched until
- * the stream reaches this work.  Calls on different streams may overlap.
- * Errors: FP_EINVAL, FP_ENOMEM (stream-ordered scratch), FP_ECUDA. */
+ * the stream reaches this work.  Calls on different streams may overlap.  A
+ * small batch may use stream-ordered scratch (a forest of one pass does
+ * without when there is none, or when the stream is being captured).
+ * Errors: FP_EINVAL, FP_ENOMEM (scratch of a forest of several passes),
+ * FP_ECUDA. */
 int fp_predict(const fp_device_forest *forest, const float *X, int64_t n, uint32_t *out_votes, int32_t *out_class,
                void *stream);
 
@@ -231,13 +239,14 @@ int fp_predict(const fp_device_forest *forest, const float *X, int64_t n, uint32
  * budget and must not grow or fragment the heap, code that runs while it
  * holds its own allocator's lock, or code that must not reach the driver's
  * allocation path, which can synchronise the device.
- * Arguments, outputs and errors are those of fp_predict.  A forest swept in
- * several passes needs scratch (a vote accumulator when out_votes is NULL and
- * one counter per observation tile when out_class is given); here it comes
- * from one fixed 16 MiB device array inside the library, which every GPU that
- * loads the library holds until the process exits.  A call whose scratch
- * would exceed 16 MiB returns FP_EINVAL before enqueuing anything (pass
- * out_votes, split the batch, or use fp_predict).  The first call on a device
+ * Arguments, outputs and errors are those of fp_predict.  A forest of several
+ * passes may need scratch (a vote accumulator and one counter per observation
+ * tile); here it comes from one fixed 16 MiB device array inside the library,
+ * which every GPU that loads the library holds until the process exits.  A
+ * call on such a forest returns FP_EINVAL before enqueuing anything when the
+ * accumulator for all rows (when out_votes is NULL) and the counters (when
+ * out_class is given) would exceed 16 MiB (pass out_votes, split the batch, or
+ * use fp_predict).  The first call on a device
  * looks up the array's device address, so make it before any CUDA-graph
  * stream capture.  All calls on a device share its one array, which keeps
  * the last call's contents; each call clears the part it uses.  Calls whose

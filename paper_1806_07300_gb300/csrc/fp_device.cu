@@ -1,11 +1,12 @@
 // fp_device.cu -- resident forests and the classification entry points.
 //
 // fp_upload copies a packed image to the device; fp_predict launches the
-// persistent traversal kernel (fp_traverse.cuh) on the caller's stream.  The
-// kernel needs scratch memory only when a forest is swept in several passes
-// (a vote accumulator when the caller asks for classes only, and one counter
-// per observation tile); that scratch comes from a library-owned
-// stream-ordered memory pool, so calls on different streams never share it.
+// persistent traversal kernel (fp_traverse.cuh) on the caller's stream, in the
+// shape that plan_rows chooses for the batch.  The kernel needs scratch memory
+// only where a forest of several passes has its bins split over CTAs (a vote
+// accumulator when the caller asks for classes only, and one counter per
+// observation tile); that scratch comes from a library-owned stream-ordered
+// memory pool, so calls on different streams never share it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,6 +35,7 @@ struct fp_device_forest {
     int32_t nbuf = 3;                          // bin-block buffers
     size_t smem_votes = 0, smem_leaves = 0, smem_values = 0;
     int32_t grid_votes = 0, grid_leaves = 0, grid_values = 0;  // resident CTAs for a persistent launch
+    double cost_fixed = 0.0, cost_row = 0.0, cost_task = 0.0;  // of an item (fit_costs)
     int32_t spin_limit = FP_SPIN_LIMIT;       // fault injection may lower it
     int32_t stall = 0;                        // fault injection: bin waits run out
 };
@@ -229,6 +231,142 @@ int launch_setup(fp_device_forest *f, int32_t tile, int32_t warps, int32_t refil
     return FP_OK;
 }
 
+// ------------------------------------------------------- shape of a launch
+//
+// A batch is cut into tiles of R rows, and a tile's bins into S splits.  Large
+// batches fill the GPU with tiles (S = 1: a CTA sweeps the whole forest for
+// its tile, the CTAs walking the same bins at about the same time, so that L2
+// serves them; 256 trees of 208 MB of super-nodes, 4 M rows: 24.8 ms, 25.4 ms
+// when swept pass by pass, for the rows staged and the votes added once per
+// pass).  A batch too small for that leaves SMs idle, or its last wave nearly
+// empty, unless the bins are split as well; the splits of a tile then add up
+// in global memory (scratch, a memset, and the last CTA's second look at the
+// tile: 3 to 4 us), where a 32-row request on 64 trees had one CTA walk 22
+// bins one after another.
+// A batch of a few waves is cut in two: the rows that fill whole waves of the
+// largest tile, and the rest in the shape that is best for it.
+
+struct Shape {
+    int32_t R = 32, S = 1;
+    double cost = 1e300;  // estimated nanoseconds
+};
+
+struct Part {
+    int64_t row0 = 0, n = 0;
+    Shape shape;
+};
+
+// Estimated time of one item, in nanoseconds, fitted to launches of one wave
+// over forests of 16 to 256 trees, tiles of 32 to 864 rows and 1 to 86 bins
+// (within 20 % for most; only the ratios matter):
+//   - what it takes before and after its walks: the first rows and blocks from
+//     memory, and the longest walks' last steps, one L2 latency each (19 us for
+//     one bin of the 256-tree forest, 29 us for one of 784-feature trees, whose
+//     heads are 4 levels);
+//   - its rows through one SM's loads;
+//   - its bins: 0.8 us in which the warps take their turn at a block, and its
+//     tasks, 0.06 ns per level in the head and 0.21 ns per level below it.
+void fit_costs(fp_device_forest *f) {
+    const FpImageHeader &h = f->hdr;
+    double levels = 1.0;  // of a tree's walk
+    for (int64_t m = h.n_internal / std::max<int32_t>(1, h.n_trees); m > 1; m >>= 1) levels += 1.4;
+    const double head = std::min(levels, h.depth + 1.0), deep = h.n_super ? levels - head : 0.0;
+    f->cost_fixed = 4000.0 + 1000.0 * deep;
+    f->cost_row = 0.08 * h.n_features;
+    f->cost_task = h.n_super ? 0.3 + 0.06 * head + 0.21 * deep : 0.06 * head;
+}
+
+double item_cost(const fp_device_forest *f, int64_t R, int64_t bins) {
+    return f->cost_fixed + f->cost_row * (double)R +
+           (double)bins * (800.0 + f->cost_task * (double)R * f->hdr.bin_size);
+}
+
+// The best shape for n rows, fewer than a few waves' worth: in one split if
+// `whole` allows it, in several (up to one per bin) if `split` does and saves
+// a fifth; `extra`: what splitting costs besides.
+Shape best_shape(const fp_device_forest *f, int64_t n, int32_t slots, bool whole, bool split, double extra) {
+    const int32_t nb = f->hdr.n_bins;
+    Shape best;
+    auto try_splits = [&](int64_t S) {
+        const int64_t room = slots / S;  // tiles at a time
+        for (int64_t w = 1; w <= 4 && room > 0; ++w) {
+            const int64_t fit = ((n + w * room - 1) / (w * room) + 31) / 32 * 32;
+            const int64_t R = std::min<int64_t>(f->R, std::max<int64_t>(32, fit));
+            const int64_t tiles = (n + R - 1) / R, turns = (tiles + room - 1) / room;
+            const double c = (double)turns * item_cost(f, R, (nb + S - 1) / S) + (S > 1 ? extra : 0.0);
+            if (c < best.cost) {
+                best.R = (int32_t)R;
+                best.S = (int32_t)S;
+                best.cost = c;
+            }
+            if (R == 32) break;
+        }
+    };
+    if (whole) try_splits(1);
+    const Shape unsplit = best;
+    if (split) {
+        for (int64_t S = 2; S < nb && S <= slots; S += 1 + S / 6) try_splits(S);
+        if (nb > 1) try_splits(nb);
+    }
+    if (whole && extra > 0.0 && best.cost > 0.8 * unsplit.cost) return unsplit;
+    return best;
+}
+
+// How n rows are launched: in one or two parts (returns how many).  split: a
+// forest of one pass may have its bins split, which takes scratch (leaf ids
+// take none).
+int plan_rows(const fp_device_forest *f, int64_t n, int32_t grid, bool split, bool leaves, Part out[2]) {
+    const FpImageHeader &h = f->hdr;
+    const int64_t wave = (int64_t)grid * f->R;  // rows of a full wave of the largest tiles
+    const bool passes = h.n_passes > 1;
+    // A forest beyond L2 whose tiles are too small to use a bin's lines before
+    // the next bin's evict them (more than 16 bytes of it per task in a wave)
+    // is swept pass by pass, all tiles of a pass before the next pass.
+    const int64_t deep = 32 * (int64_t)h.n_super;
+    if (passes && deep > ((int64_t)96 << 20) && deep > 16 * wave * h.n_trees) {
+        const int64_t want = (n * h.n_passes + grid - 1) / grid;
+        out[0].row0 = 0;
+        out[0].n = n;
+        out[0].shape = Shape();
+        out[0].shape.R = (int32_t)std::min<int64_t>(f->R, std::max<int64_t>(32, (want + 31) / 32 * 32));
+        out[0].shape.S = h.n_passes;
+        return 1;
+    }
+    auto small = [&](int64_t m) {  // the best shape for less than a few waves
+        if (leaves) return best_shape(f, m, grid, true, true, 0.0);
+        // a forest of several passes has bins enough to split: it is kept
+        // whole only for rows that fill the GPU with two slabs per CTA
+        if (passes) return best_shape(f, m, grid, m >= 64 * (int64_t)grid, true, 4000.0);
+        return best_shape(f, m, grid, true, split, 4000.0);
+    };
+    const int64_t full = n / wave;
+    if (full == 0) {
+        out[0].row0 = 0;
+        out[0].n = n;
+        out[0].shape = small(n);
+        return 1;
+    }
+    // whole waves only, in tiles as even as 32-row steps allow ...
+    const int64_t waves = (n + wave - 1) / wave;
+    Shape even;
+    even.R = (int32_t)std::min<int64_t>(f->R, ((n + waves * grid - 1) / (waves * grid) + 31) / 32 * 32);
+    even.cost = (double)(((n + even.R - 1) / even.R + grid - 1) / grid) * item_cost(f, even.R, h.n_bins);
+    out[0].row0 = 0;
+    out[0].n = n;
+    out[0].shape = even;
+    const int64_t rest = n - full * wave;
+    if (rest == 0) return 1;
+    // ... or full waves and the rest apart
+    const Shape tail = small(rest);
+    if ((double)full * item_cost(f, f->R, h.n_bins) + tail.cost + 8000.0 >= even.cost) return 1;
+    out[0].n = full * wave;
+    out[0].shape.R = f->R;
+    out[1].row0 = full * wave;
+    out[1].n = rest;
+    out[1].shape = tail;
+    return 2;
+}
+
 TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
     TravParams p;
     memset(&p, 0, sizeof p);
@@ -244,16 +382,14 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
     p.F = h.n_features;
     p.C = h.n_classes;
     p.T = h.n_trees;
-    // A small batch gets smaller tiles, so that its (pass, tile) items still
-    // reach every resident CTA; shared memory is laid out for f->R rows and a
-    // smaller tile (a multiple of 32) fits in it.
-    int32_t R = f->R;
-    const int64_t grid = std::max<int64_t>(1, f->grid_votes);
-    const int64_t want = (n * std::max<int32_t>(1, h.n_passes) + grid - 1) / grid;  // rows per tile
-    if (want < R) R = (int32_t)std::max<int64_t>(32, (want + 31) / 32 * 32);
-    p.R = R;
+    p.R = f->R;
     p.slab = (uint32_t)slab_bytes(h.n_features, h.n_classes, false);  // other modes set their own
-    p.n_tiles = (n + R - 1) / R;
+    p.n_tiles = (n + p.R - 1) / p.R;
+    p.n_items = p.n_tiles;
+    p.n_splits = 1;
+    p.n_passes = h.n_passes;
+    p.n_bins = h.n_bins;
+    p.split_bins = h.n_bins;
     p.head_smem = f->head_smem;
     p.nbuf = f->nbuf;
     p.levels = h.head_select == 3 ? 0 : h.head_select;  // kernel: 0 ranked, 1 level slots, 2 paired
@@ -285,6 +421,40 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
         p.deep_keys = reinterpret_cast<const uint32_t *>(f->d_image + h.off_deep_keys);
     }
     return p;
+}
+
+void set_shape(TravParams &p, const Shape &sh) {
+    p.R = sh.R;
+    p.n_tiles = (p.n + sh.R - 1) / sh.R;
+    p.n_splits = sh.S;
+    p.n_items = p.n_tiles * sh.S;
+    p.split_bins = p.n_bins / sh.S;
+    p.split_more = p.n_bins % sh.S;
+}
+
+// Launch one part of a call, shaped by set_shape.
+template <int MODE>
+cudaError_t launch_part(const fp_device_forest *f, const TravParams &p, int32_t grid, size_t smem, cudaStream_t s) {
+    const int64_t ctas = std::min<int64_t>(p.n_items, grid);
+    traverse_kernel<MODE>(f)<<<(unsigned)ctas, f->threads, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
+// Whether a call on this stream may take scratch that it would not need
+// otherwise: while the stream is captured it becomes a memory node, which
+// limits what can be done with the graph.
+bool may_split(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+}
+
+// Scratch of a part whose splits add up in global memory: acc_per_row bytes of
+// accumulator per row, then a counter per tile.
+size_t scratch_bytes(const Part &pt, int64_t acc_per_row, size_t *acc_bytes) {
+    *acc_bytes = 0;
+    if (pt.shape.S == 1) return 0;
+    *acc_bytes = ((size_t)pt.n * acc_per_row + 255) & ~(size_t)255;
+    return *acc_bytes + (size_t)((pt.n + pt.shape.R - 1) / pt.shape.R) * 4;
 }
 
 int check_device(const fp_device_forest *f) {
@@ -342,6 +512,7 @@ extern "C" int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_for
     e = cudaStreamSynchronize(s);  // the caller may free the host image on return
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaStreamSynchronize"); goto fail; }
     f->head_smem = (h->max_head_bytes + 15) & ~15;
+    fit_costs(f);
     rc = launch_setup(f, h->obs_tile, h->warps_per_cta, h->refill_lanes, h->bin_buffers);
     if (rc) goto fail;
     *out = f;
@@ -373,6 +544,53 @@ extern "C" int fp_configure(fp_device_forest *f, const fp_pack_params *params) {
                         params->bin_buffers ? params->bin_buffers : f->nbuf);
 }
 
+namespace {
+
+// fp_predict and fp_predict_noalloc: scratch_for(bytes, &ptr) supplies the
+// scratch of a part, release(ptr) takes it back.  A part that gets none runs
+// unsplit where the forest has one pass, or where `whole` says so.
+template <class Scratch, class Release>
+int predict_votes(const fp_device_forest *f, const float *X, int64_t n, uint32_t *out_votes, int32_t *out_class,
+                  cudaStream_t s, bool split, bool whole, Scratch scratch_for, Release release) {
+    const FpImageHeader &h = f->hdr;
+    Part parts[2];
+    const int k = plan_rows(f, n, f->grid_votes, split, false, parts);
+    for (int i = 0; i < k; ++i) {
+        Part &pt = parts[i];
+        uint32_t *const votes = out_votes ? out_votes + pt.row0 * h.n_classes : nullptr;
+        // the splits add up in scratch, or, where that would be large, in the
+        // caller's votes (a second memset)
+        const int64_t vote_bytes = 4 * (int64_t)h.n_classes;
+        const bool in_votes = votes && pt.n * vote_bytes > (4 << 20);
+        size_t acc_bytes;
+        const size_t bytes = scratch_bytes(pt, in_votes ? 0 : vote_bytes, &acc_bytes);
+        void *scratch = nullptr;
+        if (bytes) {
+            const int rc = scratch_for(bytes, &scratch);
+            if (rc && h.n_passes > 1 && !whole) return rc;
+            if (rc) pt.shape.S = 1;  // the same rows without scratch
+        }
+        TravParams p = base_params(f, X + pt.row0 * h.n_features, pt.n);
+        set_shape(p, pt.shape);
+        p.out_votes = votes;
+        p.out_class = out_class ? out_class + pt.row0 : nullptr;
+        cudaError_t e = cudaSuccess;
+        if (p.n_splits > 1) {
+            uint8_t *sc = static_cast<uint8_t *>(scratch);
+            p.acc = in_votes ? votes : reinterpret_cast<uint32_t *>(sc);
+            p.tile_done = reinterpret_cast<uint32_t *>(sc + acc_bytes);
+            e = cudaMemsetAsync(scratch, 0, bytes, s);
+            if (e == cudaSuccess && in_votes) e = cudaMemsetAsync(votes, 0, (size_t)(pt.n * vote_bytes), s);
+        }
+        if (e == cudaSuccess) e = launch_part<FP_MODE_VOTES>(f, p, f->grid_votes, f->smem_votes, s);
+        if (scratch) release(scratch);
+        if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel launch");
+    }
+    return FP_OK;
+}
+
+}  // namespace
+
 extern "C" int fp_predict(const fp_device_forest *f, const float *X, int64_t n, uint32_t *out_votes,
                           int32_t *out_class, void *stream) {
     if (!f || n < 0 || (n > 0 && !X)) {
@@ -387,41 +605,10 @@ extern "C" int fp_predict(const fp_device_forest *f, const float *X, int64_t n, 
     int rc = check_device(f);
     if (rc) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const FpImageHeader &h = f->hdr;
-    TravParams p = base_params(f, X, n);
-    p.n_passes = h.n_passes;
-    p.n_items = p.n_tiles * h.n_passes;
-    p.out_votes = out_votes;
-    p.out_class = out_class;
-    void *scratch = nullptr;
-    cudaError_t e;
-    if (h.n_passes > 1) {
-        const size_t vote_bytes = out_votes ? 0 : (size_t)n * h.n_classes * 4;
-        const size_t cnt_bytes = out_class ? (size_t)p.n_tiles * 4 : 0;
-        const size_t bytes = ((vote_bytes + 255) & ~(size_t)255) + cnt_bytes;
-        if (bytes) {
-            rc = scratch_alloc(f->device, &scratch, bytes, s);
-            if (rc) return rc;
-            e = cudaMemsetAsync(scratch, 0, bytes, s);
-            if (e != cudaSuccess) { cudaFreeAsync(scratch, s); return cuda_fail(e, "cudaMemsetAsync(scratch)"); }
-        }
-        uint8_t *sc = static_cast<uint8_t *>(scratch);
-        p.acc = out_votes ? out_votes : reinterpret_cast<uint32_t *>(sc);
-        p.tile_done = reinterpret_cast<uint32_t *>(sc + ((vote_bytes + 255) & ~(size_t)255));
-        if (out_votes) {
-            e = cudaMemsetAsync(out_votes, 0, (size_t)n * h.n_classes * 4, s);
-            if (e != cudaSuccess) {
-                if (scratch) cudaFreeAsync(scratch, s);
-                return cuda_fail(e, "cudaMemsetAsync(out_votes)");
-            }
-        }
-    }
-    const int64_t grid = std::min<int64_t>(p.n_items, f->grid_votes);
-    traverse_kernel<FP_MODE_VOTES>(f)<<<(unsigned)grid, f->threads, f->smem_votes, s>>>(p);
-    e = cudaGetLastError();
-    if (scratch) cudaFreeAsync(scratch, s);
-    if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel launch");
-    return FP_OK;
+    return predict_votes(
+        f, X, n, out_votes, out_class, s, may_split(s), false,
+        [&](size_t bytes, void **out) { return scratch_alloc(f->device, out, bytes, s); },
+        [&](void *ptr) { cudaFreeAsync(ptr, s); });
 }
 
 extern "C" int fp_predict_values(const fp_device_forest *f, const float *X, int64_t n, float scale, float bias,
@@ -439,31 +626,34 @@ extern "C" int fp_predict_values(const fp_device_forest *f, const float *X, int6
     if (rc) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const FpImageHeader &h = f->hdr;
-    TravParams p = base_params(f, X, n);
-    p.n_passes = h.n_passes;
-    p.n_items = p.n_tiles * h.n_passes;
-    p.slab = (uint32_t)slab_bytes(h.n_features, 1, false);
-    p.vscale = scale;
-    p.vbias = bias;
-    p.out_val = out;
-    void *scratch = nullptr;
-    cudaError_t e;
-    if (h.n_passes > 1) {  // a float accumulator per row and a counter per tile
-        const size_t acc_bytes = ((size_t)n * 4 + 255) & ~(size_t)255;
-        const size_t bytes = acc_bytes + (size_t)p.n_tiles * 4;
-        rc = scratch_alloc(f->device, &scratch, bytes, s);
-        if (rc) return rc;
-        e = cudaMemsetAsync(scratch, 0, bytes, s);
-        if (e != cudaSuccess) { cudaFreeAsync(scratch, s); return cuda_fail(e, "cudaMemsetAsync(scratch)"); }
-        uint8_t *sc = static_cast<uint8_t *>(scratch);
-        p.acc_val = reinterpret_cast<float *>(sc);
-        p.tile_done = reinterpret_cast<uint32_t *>(sc + acc_bytes);
+    Part parts[2];
+    const int k = plan_rows(f, n, f->grid_values, may_split(s), false, parts);
+    for (int i = 0; i < k; ++i) {
+        Part &pt = parts[i];
+        size_t acc_bytes;  // a float accumulator per row, a counter per tile
+        const size_t bytes = scratch_bytes(pt, 4, &acc_bytes);
+        void *scratch = nullptr;
+        if (bytes) {
+            rc = scratch_alloc(f->device, &scratch, bytes, s);
+            if (rc && h.n_passes > 1) return rc;
+            if (rc) pt.shape.S = 1;  // the same rows without scratch
+        }
+        TravParams p = base_params(f, X + pt.row0 * h.n_features, pt.n);
+        set_shape(p, pt.shape);
+        p.slab = (uint32_t)slab_bytes(h.n_features, 1, false);
+        p.vscale = scale;
+        p.vbias = bias;
+        p.out_val = out + pt.row0;
+        cudaError_t e = cudaSuccess;
+        if (p.n_splits > 1) {
+            e = cudaMemsetAsync(scratch, 0, bytes, s);
+            p.acc_val = static_cast<float *>(scratch);
+            p.tile_done = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(scratch) + acc_bytes);
+        }
+        if (e == cudaSuccess) e = launch_part<FP_MODE_VALUES>(f, p, f->grid_values, f->smem_values, s);
+        if (scratch) cudaFreeAsync(scratch, s);
+        if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel<values> launch");
     }
-    const int64_t grid = std::min<int64_t>(p.n_items, f->grid_values);
-    traverse_kernel<FP_MODE_VALUES>(f)<<<(unsigned)grid, f->threads, f->smem_values, s>>>(p);
-    e = cudaGetLastError();
-    if (scratch) cudaFreeAsync(scratch, s);
-    if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel<values> launch");
     return FP_OK;
 }
 
@@ -512,15 +702,13 @@ extern "C" int fp_predict_noalloc(const fp_device_forest *f, const float *X, int
     if (rc) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const FpImageHeader &h = f->hdr;
-    TravParams p = base_params(f, X, n);
-    p.n_passes = h.n_passes;
-    p.n_items = p.n_tiles * h.n_passes;
-    p.out_votes = out_votes;
-    p.out_class = out_class;
-    cudaError_t e;
     if (h.n_passes > 1) {
+        // the documented limit: a vote accumulator and tile counters for the
+        // whole batch, with tiles small enough that every pass fills the GPU
+        const int64_t grid = std::max<int64_t>(1, f->grid_votes), want = (n * h.n_passes + grid - 1) / grid;
+        const int64_t R = std::min<int64_t>(f->R, std::max<int64_t>(32, (want + 31) / 32 * 32));
         const size_t vote_bytes = out_votes ? 0 : (size_t)n * h.n_classes * 4;
-        const size_t cnt_bytes = out_class ? (size_t)p.n_tiles * 4 : 0;
+        const size_t cnt_bytes = out_class ? (size_t)((n + R - 1) / R) * 4 : 0;
         const size_t bytes = ((vote_bytes + 255) & ~(size_t)255) + cnt_bytes;
         if (bytes > FP_NOALLOC_SCRATCH_BYTES) {
             fp_set_error("fp_predict_noalloc: %lld rows need %zu bytes of scratch, more than the fixed %u; pass "
@@ -528,26 +716,18 @@ extern "C" int fp_predict_noalloc(const fp_device_forest *f, const float *X, int
                          (long long)n, bytes, FP_NOALLOC_SCRATCH_BYTES);
             return FP_EINVAL;
         }
-        void *scratch = nullptr;
-        rc = noalloc_scratch(f->device, &scratch);
-        if (rc) return rc;
-        if (bytes) {
-            e = cudaMemsetAsync(scratch, 0, bytes, s);  // the last call's counts must not leak in
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(noalloc scratch)");
-        }
-        uint8_t *sc = static_cast<uint8_t *>(scratch);
-        p.acc = out_votes ? out_votes : reinterpret_cast<uint32_t *>(sc);
-        p.tile_done = reinterpret_cast<uint32_t *>(sc + ((vote_bytes + 255) & ~(size_t)255));
-        if (out_votes) {
-            e = cudaMemsetAsync(out_votes, 0, (size_t)n * h.n_classes * 4, s);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync(out_votes)");
-        }
     }
-    const int64_t grid = std::min<int64_t>(p.n_items, f->grid_votes);
-    traverse_kernel<FP_MODE_VOTES>(f)<<<(unsigned)grid, f->threads, f->smem_votes, s>>>(p);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel launch");
-    return FP_OK;
+    return predict_votes(
+        f, X, n, out_votes, out_class, s, false, true,
+        [&](size_t bytes, void **out) {
+            if (bytes > FP_NOALLOC_SCRATCH_BYTES) {
+                fp_set_error("fp_predict_noalloc: %zu bytes of scratch, more than the fixed %u", bytes,
+                             FP_NOALLOC_SCRATCH_BYTES);
+                return FP_EINVAL;
+            }
+            return noalloc_scratch(f->device, out);
+        },
+        [](void *) {});
 }
 
 extern "C" int fp_predict_leaves(const fp_device_forest *f, const float *X, int64_t n, int32_t *out_leaf,
@@ -560,15 +740,17 @@ extern "C" int fp_predict_leaves(const fp_device_forest *f, const float *X, int6
     int rc = check_device(f);
     if (rc) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    TravParams p = base_params(f, X, n);
-    p.n_passes = f->hdr.n_passes;
-    p.n_items = p.n_tiles * f->hdr.n_passes;
-    p.slab = (uint32_t)slab_bytes(f->hdr.n_features, 0, true);
-    p.out_leaf = out_leaf;
-    const int64_t grid = std::min<int64_t>(p.n_items, f->grid_leaves);
-    traverse_kernel<FP_MODE_LEAVES>(f)<<<(unsigned)grid, f->threads, f->smem_leaves, s>>>(p);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel<leaves> launch");
+    Part parts[2];
+    const int k = plan_rows(f, n, f->grid_leaves, false, true, parts);
+    for (int i = 0; i < k; ++i) {
+        const Part &pt = parts[i];
+        TravParams p = base_params(f, X + pt.row0 * f->hdr.n_features, pt.n);
+        set_shape(p, pt.shape);
+        p.slab = (uint32_t)slab_bytes(f->hdr.n_features, 0, true);
+        p.out_leaf = out_leaf + pt.row0 * f->hdr.n_trees;
+        cudaError_t e = launch_part<FP_MODE_LEAVES>(f, p, f->grid_leaves, f->smem_leaves, s);
+        if (e != cudaSuccess) return cuda_fail(e, "fp_traverse_kernel<leaves> launch");
+    }
     return FP_OK;
 }
 
@@ -638,7 +820,38 @@ extern "C" void fp_release(fp_device_forest *f) {
     delete f;
 }
 
-// One persistent launch over up to FP_MAX_BATCH (forest, batch) pairs.
+// The shape of one batch when no item of it is to take longer than `most`
+// nanoseconds: the splits, of a few numbers of them, whose items (as large as
+// `most` lets them be) take the least time together.
+static Shape shape_within(const fp_device_forest *f, int64_t n, int32_t max_R, double most) {
+    const int64_t nb = f->hdr.n_bins, top = std::min<int64_t>(max_R, (n + 31) / 32 * 32);
+    Shape best;
+    for (int64_t S = 1;; S = std::min(nb, S + 1 + S / 2)) {
+        const int64_t bins = (nb + S - 1) / S;
+        const double fixed = item_cost(f, 0, bins), per_row = item_cost(f, 1, bins) - fixed;
+        const double fit = std::max(32.0, std::min((most - fixed) / per_row, (double)top));
+        const int64_t R = (int64_t)fit / 32 * 32, tiles = (n + R - 1) / R;
+        const double item = item_cost(f, R, bins) + (S > 1 ? 1000.0 : 0.0);
+        // an item that is too long all the same counts for more
+        const double cost = (double)(tiles * S) * item * (item > most ? item / most : 1.0);
+        if (cost < best.cost) {
+            best.R = (int32_t)R;
+            best.S = (int32_t)S;
+            best.cost = cost;
+        }
+        if (S == nb) break;
+    }
+    return best;
+}
+
+// One persistent launch over up to FP_MAX_BATCH (forest, batch) pairs.  How
+// long an item may take is chosen for the whole launch: of a few lengths, the
+// one with the least estimated end: the longest item when all items run at
+// once, else the items' sum over the GPU's CTAs and the longest item besides
+// (it may begin last).  Tiles as large as each forest's
+// own left the last of them running alone, and a batch of a few rows walked
+// all bins of a pass in one CTA (four forests, 3 to 52,001 rows: 379 us; four
+// of 33 to 178 rows: 76 us).
 static int predict_batched_chunk(const fp_device_forest *const *forests, const fp_batch *batches, int32_t k,
                                  cudaStream_t s) {
     int device = -1;
@@ -651,11 +864,14 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
     int warps = 1;
     for (int32_t j = 0; j < k; ++j) warps = std::max(warps, forests[j]->threads / 32);
 
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
+
     BatchParams bp;
     memset(&bp, 0, sizeof bp);
     size_t smem = 0;
-    size_t scratch_bytes = 256;  // the work counter, then per-batch accumulators and tile counters
-    std::vector<size_t> acc_off((size_t)k, 0), cnt_off((size_t)k, 0);
+    int32_t live[FP_MAX_BATCH], max_R[FP_MAX_BATCH];  // batches with work, and their largest tiles
     int32_t m = 0;
     for (int32_t j = 0; j < k; ++j) {
         const fp_device_forest *f = forests[j];
@@ -670,31 +886,50 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
             return FP_EUNSUPPORTED;
         }
         smem = std::max(smem, need);
+        live[m] = j;
+        max_R[m++] = R;
+    }
+    if (m == 0) return FP_OK;
+    double best_end = 1e300, most = 0.0;
+    for (double len = 8000.0; len < 4e6; len *= 1.5) {
+        double sum = 0.0, longest = 0.0, items = 0.0;
+        for (int32_t i = 0; i < m; ++i) {
+            const fp_device_forest *f = forests[live[i]];
+            const Shape sh = shape_within(f, batches[live[i]].n, max_R[i], len);
+            const double item = item_cost(f, sh.R, (f->hdr.n_bins + sh.S - 1) / sh.S);
+            const double count = (double)((batches[live[i]].n + sh.R - 1) / sh.R * sh.S);
+            sum += item * count;
+            items += count;
+            longest = std::max(longest, item);
+        }
+        const double end = items <= sms ? longest : sum / sms + longest;
+        if (end < best_end) {
+            best_end = end;
+            most = len;
+        }
+    }
+    size_t scratch_bytes = 256;  // the work counter, then per-batch accumulators and tile counters
+    size_t acc_off[FP_MAX_BATCH] = {0}, cnt_off[FP_MAX_BATCH] = {0};
+    for (int32_t i = 0; i < m; ++i) {
+        const fp_device_forest *f = forests[live[i]];
+        const fp_batch &bt = batches[live[i]];
         TravParams p = base_params(f, bt.X, bt.n);
-        p.R = R;
-        p.n_tiles = (bt.n + R - 1) / R;
-        p.n_passes = h.n_passes;
-        p.n_items = p.n_tiles * h.n_passes;
+        set_shape(p, shape_within(f, bt.n, max_R[i], most));
         p.out_votes = bt.out_votes;
         p.out_class = bt.out_class;
-        if (h.n_passes > 1) {
-            if (!bt.out_votes) {
-                acc_off[j] = scratch_bytes;
-                scratch_bytes += ((size_t)bt.n * h.n_classes * 4 + 255) & ~(size_t)255;
+        if (p.n_splits > 1) {
+            const size_t votes = (size_t)bt.n * f->hdr.n_classes * 4;
+            if (!bt.out_votes || votes <= (4u << 20)) {  // else they add up in the caller's votes
+                acc_off[i] = scratch_bytes;
+                scratch_bytes += (votes + 255) & ~(size_t)255;
             }
-            if (bt.out_class) {
-                cnt_off[j] = scratch_bytes;
-                scratch_bytes += ((size_t)p.n_tiles * 4 + 255) & ~(size_t)255;
-            }
+            cnt_off[i] = scratch_bytes;
+            scratch_bytes += ((size_t)p.n_tiles * 4 + 255) & ~(size_t)255;
         }
-        bp.p[m] = p;
-        acc_off[m] = acc_off[j];
-        cnt_off[m] = cnt_off[j];
-        bp.item_begin[m + 1] = bp.item_begin[m] + p.n_items;
-        ++m;
+        bp.p[i] = p;
+        bp.item_begin[i + 1] = bp.item_begin[i] + p.n_items;
     }
     bp.k = m;
-    if (m == 0) return FP_OK;
     void *scratch = nullptr;
     int rc = scratch_alloc(device, &scratch, scratch_bytes, s);
     if (rc) return rc;
@@ -702,10 +937,10 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
     e = cudaMemsetAsync(scratch, 0, scratch_bytes, s);
     for (int32_t j = 0; j < m && e == cudaSuccess; ++j) {
         TravParams &p = bp.p[j];
-        if (p.n_passes > 1) {
-            p.acc = p.out_votes ? p.out_votes : reinterpret_cast<uint32_t *>(sc + acc_off[j]);
-            if (p.out_class) p.tile_done = reinterpret_cast<uint32_t *>(sc + cnt_off[j]);
-            if (p.out_votes) e = cudaMemsetAsync(p.out_votes, 0, (size_t)p.n * p.C * 4, s);
+        if (p.n_splits > 1) {
+            p.acc = acc_off[j] ? reinterpret_cast<uint32_t *>(sc + acc_off[j]) : p.out_votes;
+            p.tile_done = reinterpret_cast<uint32_t *>(sc + cnt_off[j]);
+            if (!acc_off[j]) e = cudaMemsetAsync(p.out_votes, 0, (size_t)p.n * p.C * 4, s);
         }
     }
     bp.work = reinterpret_cast<unsigned long long *>(sc);
@@ -717,9 +952,8 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
         if (bp.p[j].levels != hk) hk = -1;
     }
     void (*kern)(BatchParams) = batched_kernel(dk, hk);
-    int per_sm = 0, sms = 0;
+    int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) {
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(bp.item_begin[m], (int64_t)per_sm * sms));
         kern<<<(unsigned)grid, 32 * warps, smem, s>>>(bp);

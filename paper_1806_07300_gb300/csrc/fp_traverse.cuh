@@ -1,10 +1,11 @@
 // fp_traverse.cuh -- the packed-forest traversal kernel (sm_103a).
 //
-// One work item = (pass, observation tile).  Items are ordered pass-major, so
-// at any moment the GPU walks the bins of one pass, whose super-nodes stay
-// resident in L2 while every tile of observations goes through them (the GPU
-// counterpart of the paper's bins bound to cores, Section III).  For an item
-// the CTA:
+// One work item = an observation tile and one of the parts (splits) that the
+// forest's bins are cut into: a single one for large batches, so that a CTA
+// sweeps all bins for its tile; the CTAs sweep the same bins at about the same
+// time, which keeps the bins' super-nodes in L2 while every tile walks them
+// (the GPU counterpart of the paper's bins bound to cores, Section III).  How
+// a call is cut up is chosen on the host (fp_device.cu).  For an item the CTA:
 //   1. stages the tile's rows into shared memory in slabs of 32 rows: a slab
 //      holds its F features and then its vote counters (one per class, or one
 //      float sum), 32 words each, row l of the slab in column l.  32 lanes
@@ -43,22 +44,21 @@
 //      warp wait for another;
 //   4. counts votes per (row, class) with shared-memory atomics;
 //   5. writes votes and the argmax class (lowest class on ties).  With one
-//      pass the tile's votes are complete in shared memory; with several, they
+//      split the tile's votes are complete in shared memory; with several, they
 //      are added to a global accumulator and the CTA that finishes a tile's
-//      last pass (per-tile counter, no waiting) takes the argmax.
+//      last split takes the argmax (per-tile counter, no waiting).
 // Parity mode writes the leaf id reached in every (observation, tree)
 // instead of voting.  Values mode (forests with real leaf values: regression
 // and boosted trees) adds the leaf's value to a float per row instead, and
-// writes bias + scale * sum (several passes: summed in global memory, the
-// last pass's CTA writes it).
+// writes bias + scale * sum (several splits: summed in global memory, the
+// last split's CTA writes it).
 //
 // What bounds it (256 trees of 78.8k nodes, 28 features, 4 M rows, bins of 5
-// trees with heads 0..9: 25.4 ms, 27.5 ms before steps were straight-line code
-// over slabs): the load/store data pipe, 77 % busy with 6.1 wavefronts per
-// (row, tree), about half of them the super-nodes' sectors and half
-// shared-memory words; 19.8 warp instructions per (row, tree) (23.4 before)
-// take 62 % of the issue slots, the ALU pipe being the busiest of the
-// arithmetic ones.
+// trees with heads 0..9: 24.4 ms; 27.5 ms as one pass of L2 after another with
+// steps of divergent branches): the load/store data pipe, 80 % busy with 6.2
+// wavefronts per (row, tree), a little over half of them the super-nodes'
+// sectors and the rest shared-memory words; 17.9 warp instructions per (row,
+// tree) (23.4 before) take 63 % of the issue slots.
 //
 // Waits: __syncthreads is a hardware wait; a wait for
 // a bin block polls its mbarrier at most spin_limit times (FP_SPIN_LIMIT
@@ -83,26 +83,30 @@ struct TravParams {
     const float *X;
     int64_t n;
     int64_t n_tiles;
-    int64_t n_items;
+    int64_t n_items;          // n_tiles * n_splits
+    int32_t n_splits;         // parts that a tile's bins are cut into, each an item of its own
+    int32_t split_bins;       // bins of a split: n_bins / n_splits, one more in the first
+    int32_t split_more;       // n_bins % n_splits
+    int32_t n_bins;
     int32_t F, C, T, R;
     uint32_t slab;            // bytes of a slab: 32 rows of F features and the mode's counters
-    int32_t n_passes;
+    int32_t n_passes;         // with as many splits, the splits are the packed passes
     int32_t head_smem;        // bytes reserved for one bin block
     int32_t nbuf;             // bin-block buffers (2 or 3)
     int32_t levels;           // head kind: 0 ranked, 1 level slots (depth+1 steps), 2 paired level slots
     int32_t depth;            // d of the interleaved head
     int32_t refill;           // bursts start when the ring holds at most this many tasks
-    uint32_t *out_votes;      // single pass: final votes (may be NULL)
+    uint32_t *out_votes;      // final votes (may be NULL, or acc)
     int32_t *out_class;       // may be NULL
     int32_t *out_leaf;        // parity mode
-    uint32_t *acc;            // several passes: vote accumulator
-    uint32_t *tile_done;      // several passes: per-tile pass counter
+    uint32_t *acc;            // several splits: vote accumulator
+    uint32_t *tile_done;      // several splits: per-tile counter of finished ones
     int32_t *status;          // device status word
     const float *leaf_val;    // forests with leaf values: value of each leaf slot
     uint32_t n_vals;          // slots in leaf_val
     float vscale, vbias;      // out = vbias + vscale * sum of leaf values
     float *out_val;           // values mode: output per row
-    float *acc_val;           // values mode, several passes: per-row accumulator
+    float *acc_val;           // values mode, several splits: per-row accumulator
     int32_t spin_limit;       // polls of a bin block's barrier before the wait gives up
     int32_t stall;            // fault injection: bin waits ignore completed copies (0 normally)
     int32_t deep_kind;        // super-nodes: 2 two levels, 3 three levels (format 1), 4 three levels (format 2)
@@ -198,22 +202,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
-// One thread: copy a bin's block into a buffer with the bulk-copy engine.
-__device__ __forceinline__ void stage_block_bulk(const TravParams &p, int b, uint8_t *dst, uint64_t *bar) {
-    const FpBin bn = p.bins[b];
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // earlier reads of dst come first
-    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)),
-                 "r"(bn.head_bytes)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-            smem_u32(dst)),
-        "l"(p.heads + bn.head_off), "r"(bn.head_bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
 // CTA-wide state shared by the items a CTA runs.
-struct CtaShared {
+struct __align__(16) CtaShared {
+    FpBin desc[FP_NBUF];      // the record of each buffer's bin
     uint64_t full[FP_NBUF];   // block staged (bulk copy done)
     int next[FP_NBUF];        // next untaken unit of the buffer's bin
     int done[FP_NBUF];        // warps done with the buffer's bin
@@ -226,27 +217,56 @@ struct CtaShared {
     long long next_item;
 };
 
-// A word of dynamic shared memory at a byte offset, by its 32-bit address
-// (through a pointer the walks took 5 to 9 % longer).
-__device__ __forceinline__ uint32_t lds(const uint8_t *smem, uint32_t off) {
+__device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+            smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
+}
+
+// Shared memory by 32-bit addresses.  The walks take theirs from one base that
+// run_item keeps in a register: through pointers to the shared arrays, the
+// compiler may form the array's address anew in every step (from a special
+// register, since it depends on the CTA's place in its cluster), which cost
+// the walks up to 9 % of their time.
+__device__ __forceinline__ uint32_t lds(uint32_t addr) {
     uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(smem_u32(smem) + off));
+    asm volatile("ld.shared.u32 %0, [%1];\n" : "=r"(v) : "r"(addr));
     return v;
 }
 
-__device__ __forceinline__ uint4 lds128(const uint8_t *smem, uint32_t off) {
+__device__ __forceinline__ uint2 lds64(uint32_t addr) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "r"(addr));
+    return v;
+}
+
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"(smem_u32(smem) + off));
+                 : "r"(addr));
     return v;
+}
+
+__device__ __forceinline__ void sts64(uint32_t addr, uint32_t x, uint32_t y) {
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};\n" ::"r"(addr), "r"(x), "r"(y) : "memory");
+}
+
+__device__ __forceinline__ void add_shared(uint32_t addr, uint32_t v) {
+    asm volatile("red.shared.add.u32 [%0], %1;\n" ::"r"(addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void add_shared(uint32_t addr, float v) {
+    asm volatile("red.shared.add.f32 [%0], %1;\n" ::"r"(addr), "f"(v) : "memory");
 }
 
 // Per-lane state of a running task.  A corrupt record only sets `bad`,
 // reported at the item's end, so that a step stays straight-line code.
 struct LaneTask {
     uint32_t ref;     // current super-node (index into deep), or FP_NO_TASK
-    uint32_t xb;      // shared-memory offset of the row: feature f is 128 f bytes further on
+    uint32_t xb;      // shared-memory address of the row: feature f is 128 f bytes further on
     uint32_t rt;      // parity mode: row within the tile | tree << 11
     int bad;
 };
@@ -264,15 +284,15 @@ struct Pending {
 // A vote for class `cls` of the row at xb.  Class 0 is not counted: its votes
 // are the item's trees less all the others'.  Returns false for a class that
 // does not exist.
-__device__ __forceinline__ bool vote(const TravParams &p, uint8_t *smem, bool on, uint32_t xb, uint32_t cls) {
+__device__ __forceinline__ bool vote(const TravParams &p, bool on, uint32_t xb, uint32_t cls) {
     const bool counted = cls - 1u < (uint32_t)p.C - 1u;
-    if (on && counted) atomicAdd(reinterpret_cast<uint32_t *>(smem + xb + (((uint32_t)p.F + cls) << 7)), 1u);
+    if (on && counted) add_shared(xb + (((uint32_t)p.F + cls) << 7), 1u);
     return !on || counted || cls == 0u;
 }
 
 // The row's sum of leaf values (values mode).
-__device__ __forceinline__ void add_value(const TravParams &p, uint8_t *smem, uint32_t xb, float v) {
-    atomicAdd(reinterpret_cast<float *>(smem + xb + ((uint32_t)p.F << 7)), v);
+__device__ __forceinline__ void add_value(const TravParams &p, uint32_t xb, float v) {
+    add_shared(xb + ((uint32_t)p.F << 7), v);
 }
 
 __device__ __forceinline__ void put_leaf(const TravParams &p, const CtaShared &sh, uint32_t rt, int32_t leaf_id) {
@@ -280,11 +300,11 @@ __device__ __forceinline__ void put_leaf(const TravParams &p, const CtaShared &s
 }
 
 template <int MODE>
-__device__ __forceinline__ void settle(const TravParams &p, uint8_t *smem, const CtaShared &sh, Pending &pend) {
+__device__ __forceinline__ void settle(const TravParams &p, const CtaShared &sh, Pending &pend) {
     if (MODE == FP_MODE_VOTES) return;
     if (pend.on) {
         if (MODE == FP_MODE_VALUES)
-            add_value(p, smem, pend.at, __uint_as_float(pend.word));
+            add_value(p, pend.at, __uint_as_float(pend.word));
         else
             put_leaf(p, sh, pend.at, (int32_t)pend.word);
     }
@@ -293,21 +313,17 @@ __device__ __forceinline__ void settle(const TravParams &p, uint8_t *smem, const
 
 // Lanes without a task take pending ones from the warp's ring.
 template <int MODE>
-__device__ __forceinline__ void pop_tasks(const TravParams &p, const uint2 *ring, int &head, int tail, LaneTask &L,
+__device__ __forceinline__ void pop_tasks(const TravParams &p, uint32_t base, uint32_t ring, int &head, int tail, LaneTask &L,
                                           unsigned lt_mask) {
     const bool free = L.ref == FP_NO_TASK;
     const unsigned idle = __ballot_sync(0xffffffffu, free);
     const int rk = __popc(idle & lt_mask);
-    if (free && rk < tail - head) {
-        const uint2 ent = ring[(head + rk) & (FP_RING - 1)];
-        L.ref = ent.x;
-        if (MODE == FP_MODE_LEAVES) {
-            L.rt = ent.y;
-            L.xb = ((ent.y & 2047u) >> 5) * p.slab + (ent.y & 31u) * 4u;
-        } else {
-            L.xb = ent.y;
-        }
-    }
+    uint32_t &second = MODE == FP_MODE_LEAVES ? L.rt : L.xb;
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %3, 0;\n @q ld.shared.v2.u32 {%0, %1}, [%2];\n}\n"
+                 : "+r"(L.ref), "+r"(second)
+                 : "r"(ring + (uint32_t)((head + rk) & (FP_RING - 1)) * 8u), "r"(free && rk < tail - head ? 1u : 0u)
+                 : "memory");
+    if (MODE == FP_MODE_LEAVES) L.xb = base + ((L.rt & 2047u) >> 5) * p.slab + (L.rt & 31u) * 4u;
     head = min(head + __popc(idle), tail);
 }
 
@@ -335,16 +351,16 @@ __device__ __forceinline__ void exit3(uint32_t ref, uint32_t w7, DeepStep &s) {
 // Three levels, format 1: full keys for the first two, and a key prefix for
 // the last, whose tie (rare) is decided by the slot's full key from the side
 // table.
-__device__ __forceinline__ DeepStep deep_step3(const TravParams &p, const uint8_t *smem, uint32_t ref, uint32_t xb,
+__device__ __forceinline__ DeepStep deep_step3(const TravParams &p, uint32_t ref, uint32_t xb,
                                                const uint32_t w[8]) {
     const uint32_t fm7 = p.fmask << 7;
-    const uint32_t k0 = lds(smem, xb + (__funnelshift_r(w[3], w[3], p.frot) & fm7));
+    const uint32_t k0 = lds(xb + (__funnelshift_r(w[3], w[3], p.frot) & fm7));
     const bool r0 = k0 > w[0];
     const uint32_t n1 = r0 ? w[2] : w[1], m1 = r0 ? w[5] : w[4];
-    const uint32_t k1 = lds(smem, xb + (__funnelshift_r(m1, m1, p.frot) & fm7));
+    const uint32_t k1 = lds(xb + (__funnelshift_r(m1, m1, p.frot) & fm7));
     const bool r1 = k1 > n1;
     const uint32_t n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
-    const uint32_t k2 = lds(smem, xb + ((n2 & p.fmask) << 7));
+    const uint32_t k2 = lds(xb + ((n2 & p.fmask) << 7));
     bool r2 = k2 > n2;  // decided by the key bits, unless they are equal
     DeepStep s;
     s.e = (r0 ? 4u : 0u) + (r1 ? 2u : 0u);
@@ -367,16 +383,16 @@ __device__ __forceinline__ DeepStep deep_step3(const TravParams &p, const uint8_
 // whole word decides the split wherever their top bits differ.  Where they
 // are equal for any of the three slots of the walk (rare), the step is taken
 // again with the slots' full keys from the side table.
-__device__ __forceinline__ DeepStep deep_step3p(const TravParams &p, const uint8_t *smem, uint32_t ref, uint32_t xb,
+__device__ __forceinline__ DeepStep deep_step3p(const TravParams &p, uint32_t ref, uint32_t xb,
                                                 const uint32_t w[8]) {
     const uint32_t fm = p.fmask;
-    const uint32_t k0 = lds(smem, xb + ((w[0] & fm) << 7));
+    const uint32_t k0 = lds(xb + ((w[0] & fm) << 7));
     bool r0 = k0 > w[0];
     uint32_t n1 = r0 ? w[2] : w[1];
-    const uint32_t k1 = lds(smem, xb + ((n1 & fm) << 7));
+    const uint32_t k1 = lds(xb + ((n1 & fm) << 7));
     bool r1 = k1 > n1;
     uint32_t n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
-    uint32_t k2 = lds(smem, xb + ((n2 & fm) << 7));
+    uint32_t k2 = lds(xb + ((n2 & fm) << 7));
     bool r2 = k2 > n2;
     // one test for the three slots, by the last level's shorter prefix: it
     // takes a few more steps again than need be
@@ -386,9 +402,9 @@ __device__ __forceinline__ DeepStep deep_step3p(const TravParams &p, const uint8
             const uint32_t *fk = p.deep_keys + 8 * (int64_t)ref;
             r0 = k0 > __ldg(fk);
             n1 = r0 ? w[2] : w[1];
-            r1 = lds(smem, xb + ((n1 & fm) << 7)) > __ldg(fk + 1 + (r0 ? 1 : 0));
+            r1 = lds(xb + ((n1 & fm) << 7)) > __ldg(fk + 1 + (r0 ? 1 : 0));
             n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
-            k2 = lds(smem, xb + ((n2 & fm) << 7));
+            k2 = lds(xb + ((n2 & fm) << 7));
             r2 = k2 > __ldg(fk + 3 + (r0 ? 2 : 0) + (r1 ? 1 : 0));
         }
         __syncwarp();
@@ -401,10 +417,10 @@ __device__ __forceinline__ DeepStep deep_step3p(const TravParams &p, const uint8
 }
 
 // Two levels, float thresholds.
-__device__ __forceinline__ DeepStep deep_step2(const uint8_t *smem, uint32_t xb, const uint32_t w[8]) {
-    const bool r0 = !goes_left<false>(lds(smem, xb + ((w[3] & 1023u) << 7)), w[0]);
+__device__ __forceinline__ DeepStep deep_step2(uint32_t xb, const uint32_t w[8]) {
+    const bool r0 = !goes_left<false>(lds(xb + ((w[3] & 1023u) << 7)), w[0]);
     const uint32_t f1 = r0 ? (w[3] >> 20) & 1023u : (w[3] >> 10) & 1023u;
-    const bool r1 = !goes_left<false>(lds(smem, xb + (f1 << 7)), r0 ? w[2] : w[1]);
+    const bool r1 = !goes_left<false>(lds(xb + (f1 << 7)), r0 ? w[2] : w[1]);
     const uint32_t x = r0 ? (r1 ? w[7] : w[6]) : (r1 ? w[5] : w[4]);
     DeepStep s;
     s.leaf = (x & FP_REF_LEAF) != 0u;
@@ -417,17 +433,20 @@ __device__ __forceinline__ DeepStep deep_step2(const uint8_t *smem, uint32_t xb,
 // DK: the forest's kind of super-node (p.deep_kind: 2, 3 or 4); a
 // compile-time choice, so no kind's step carries another's code.
 template <int MODE, int DK>
-__device__ __forceinline__ void deep_finish(const TravParams &p, uint8_t *smem, LaneTask &L, Pending &pend,
+__device__ __forceinline__ void deep_finish(const TravParams &p, LaneTask &L, Pending &pend,
                                             const uint32_t w[8]) {
     const uint32_t ref = L.ref;
     const bool on = ref != FP_NO_TASK;
-    const DeepStep s = DK == 3   ? deep_step3(p, smem, ref, L.xb, w)
-                       : DK == 4 ? deep_step3p(p, smem, ref, L.xb, w)
-                                 : deep_step2(smem, L.xb, w);
+    const DeepStep s = DK == 3   ? deep_step3(p, ref, L.xb, w)
+                       : DK == 4 ? deep_step3p(p, ref, L.xb, w)
+                                 : deep_step2(L.xb, w);
     const bool leaf = on && s.leaf;
     if (MODE == FP_MODE_VOTES) {
         const uint32_t c1 = s.cls - 1u, nc = (uint32_t)p.C - 1u;
-        if (leaf && c1 < nc) atomicAdd(reinterpret_cast<uint32_t *>(smem + L.xb + (((uint32_t)p.F + s.cls) << 7)), 1u);
+        asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %1, 0;\n @q red.shared.add.u32 [%0], 1;\n}\n" ::"r"(
+                         L.xb + (((uint32_t)p.F + s.cls) << 7)),
+                     "r"(leaf && c1 < nc ? 1u : 0u)
+                     : "memory");
         if (leaf && s.cls > nc) L.bad = 1;
     } else if (MODE == FP_MODE_VALUES) {  // start the read of the leaf's value ...
         const uint32_t slot = DK == 2 ? s.cls : p.vbase3 + 8 * ref + s.e;
@@ -451,8 +470,8 @@ __device__ __forceinline__ void deep_finish(const TravParams &p, uint8_t *smem, 
 }
 
 // The walk of one row (at xb) through the head of tree column k of the bin
-// block at offset blk, whose exits begin at `exits`: the offset of the exit
-// word it ends on, or FP_NO_EXIT (corrupt ranked heads only).  HK: the head
+// block at blk, whose exits begin at `exits`: the address of the exit word it
+// ends on, or FP_NO_EXIT (corrupt ranked heads only).  HK: the head
 // kind when known at compile time (0 ranked, 1 level slots, 2 paired level
 // slots), or -1 to read it from p.levels (the batched kernel, whose forests
 // may differ).  Record q of a level head lies at at0 + q * rec and exit e
@@ -461,7 +480,7 @@ __device__ __forceinline__ void deep_finish(const TravParams &p, uint8_t *smem, 
 #define FP_NO_EXIT 0xFFFFFFFFu
 
 template <bool KEYS, int HK>
-__device__ __forceinline__ uint32_t head_walk(const TravParams &p, const uint8_t *smem, uint32_t blk, uint32_t exits,
+__device__ __forceinline__ uint32_t head_walk(const TravParams &p, uint32_t blk, uint32_t exits,
                                               int k, int stride, int nranks, int nexits, uint32_t xb, bool my) {
     const int levels = HK >= 0 ? HK : p.levels;
     if (levels == 2) {
@@ -472,10 +491,10 @@ __device__ __forceinline__ uint32_t head_walk(const TravParams &p, const uint8_t
         uint32_t at = at0;
 #pragma unroll 1  // measured: unrolling the head walk only adds instructions
         for (int l = 0; l <= p.depth; l += 2) {
-            const uint4 nd = lds128(smem, at);
-            const bool r0 = !goes_left<KEYS>(lds(smem, xb + ((nd.w & 1023u) << 7)), nd.x);
+            const uint4 nd = lds128(at);
+            const bool r0 = !goes_left<KEYS>(lds(xb + ((nd.w & 1023u) << 7)), nd.x);
             const uint32_t f1 = nd.w >> (r0 ? 20 - 7 : 10 - 7);
-            const bool r1 = !goes_left<KEYS>(lds(smem, xb + (f1 & (1023u << 7))), r0 ? nd.z : nd.y);
+            const bool r1 = !goes_left<KEYS>(lds(xb + (f1 & (1023u << 7))), r0 ? nd.z : nd.y);
             at = 4u * at + (r0 ? right : left) + (r1 ? rec : 0u);
         }
         return exits + ((at - exits) >> 2);
@@ -487,21 +506,21 @@ __device__ __forceinline__ uint32_t head_walk(const TravParams &p, const uint8_t
         uint32_t at = at0;
 #pragma unroll 1
         for (int l = 0; l <= p.depth; ++l) {
-            const uint2 nd = *reinterpret_cast<const uint2 *>(smem + at);
-            at = 2u * at + (goes_left<KEYS>(lds(smem, xb + ((nd.y >> 22) << 7)), nd.x) ? left : right);
+            const uint2 nd = lds64(at);
+            at = 2u * at + (goes_left<KEYS>(lds(xb + ((nd.y >> 22) << 7)), nd.x) ? left : right);
         }
         return exits + ((at - exits) >> 1);
     }
-    const uint2 *hn = reinterpret_cast<const uint2 *>(smem + blk) + k;  // this tree's column of the block
+    const uint32_t hn = blk + (uint32_t)k * 8u, rec = (uint32_t)stride * 8u;  // this tree's column of the block
     uint32_t hr = 0;  // head rank, then nranks + exit index
     bool busy = my;
     while (__any_sync(0xffffffffu, busy)) {  // ranked heads: until the last lane leaves
 #pragma unroll
         for (int u = 0; u < 2; ++u) {  // two steps per vote
             if (busy) {
-                const uint2 nd = hn[hr * stride];
+                const uint2 nd = lds64(hn + hr * rec);
                 const uint32_t m = nd.y;
-                uint32_t nh = goes_left<KEYS>(lds(smem, xb + ((m >> 22) << 7)), nd.x)
+                uint32_t nh = goes_left<KEYS>(lds(xb + ((m >> 22) << 7)), nd.x)
                                   ? (m & FP_TARGET_MASK)
                                   : ((m >> FP_TARGET_BITS) & FP_TARGET_MASK);
                 busy = nh < (uint32_t)nranks;
@@ -527,7 +546,7 @@ __device__ __forceinline__ uint32_t head_walk(const TravParams &p, const uint8_t
 // value from global memory and an atomic (256 boosted trees of six levels, 2 M
 // rows: 2.93 ms as bursts, 1.53 ms as runs; bound by instruction issue).
 template <int MODE, bool KEYS, int HK>
-__device__ __forceinline__ void walk_heads(const TravParams &p, uint8_t *smem, CtaShared &sh, const FpBin &bn,
+__device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, CtaShared &sh, const FpBin &bn,
                                            uint32_t blk, uint32_t exits, int buf, int rows, int G, uint32_t inv_g,
                                            int &bad) {
     const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -540,38 +559,55 @@ __device__ __forceinline__ void walk_heads(const TravParams &p, uint8_t *smem, C
         unit = __shfl_sync(0xffffffffu, unit, 0);
         if (unit >= units) break;
         const int c = G > 1 ? (int)__umulhi((uint32_t)unit, inv_g) : unit, g = unit - c * G;
-        const uint32_t xb = (uint32_t)g * p.slab + (uint32_t)lane * 4u;
+        const uint32_t xb = base + (uint32_t)g * p.slab + (uint32_t)lane * 4u;
         const int r = g * 32 + lane;
         const bool my = r < rows;
         const int k1 = min(bn.width, (c + 1) * run);
         float sum = 0.0f;
         uint32_t ones = 0;
         for (int k = c * run; k < k1; ++k) {
-            const uint32_t at = head_walk<KEYS, HK>(p, smem, blk, exits, k, bn.stride, bn.nranks, bn.nexits, xb, my);
+            const uint32_t at = head_walk<KEYS, HK>(p, blk, exits, k, bn.stride, bn.nranks, bn.nexits, xb, my);
             if (HK <= 0 && at == FP_NO_EXIT) {
                 bad |= my;
                 continue;
             }
             if (MODE == FP_MODE_VALUES) {
-                sum += __uint_as_float(lds(smem, at));  // the exits hold the leaves' values themselves
+                sum += __uint_as_float(lds(at));  // the exits hold the leaves' values themselves
             } else if (MODE == FP_MODE_LEAVES) {
                 if (my)
                     put_leaf(p, sh, (uint32_t)r | ((uint32_t)(bn.first_tree + k) << 11),
                              p.pheads[(bn.phead_off >> 2) + ((at - exits) >> 2)]);
             } else {
-                const uint32_t cls = lds(smem, at) & 0x7FFFFFFFu;
+                const uint32_t cls = lds(at) & 0x7FFFFFFFu;
                 if (p.C == 2) {
                     ones += cls & 1u;
                     bad |= my && cls > 1u;
                 } else {
-                    bad |= !vote(p, smem, my, xb, cls);
+                    bad |= !vote(p, my, xb, cls);
                 }
             }
         }
-        if (MODE == FP_MODE_VALUES && my) add_value(p, smem, xb, sum);
+        if (MODE == FP_MODE_VALUES && my) add_value(p, xb, sum);
         if (MODE == FP_MODE_VOTES && my && p.C == 2 && ones)
-            atomicAdd(reinterpret_cast<uint32_t *>(smem + xb + (((uint32_t)p.F + 1u) << 7)), ones);
+            add_shared(xb + (((uint32_t)p.F + 1u) << 7), ones);
     }
+}
+
+// One thread: copy bin b's block (its record: bn) into a buffer with the
+// bulk-copy engine, and its record beside it, so that the warps that walk the
+// bin do not wait for that from global memory once more.
+__device__ __forceinline__ void stage_bin(const TravParams &p, CtaShared &sh, int b, const FpBin &bn, int buf,
+                                          uint8_t *dst) {
+    sh.next[buf] = 0;
+    sh.done[buf] = 0;
+    sh.issued[buf] += 1;
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // earlier reads of dst come first
+    asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;\n" ::"r"(
+                     smem_u32(&sh.full[buf])),
+                 "r"(bn.head_bytes + (uint32_t)sizeof(FpBin))
+                 : "memory");
+    bulk_copy(dst, p.heads + bn.head_off, bn.head_bytes, &sh.full[buf]);
+    bulk_copy(&sh.desc[buf], p.bins + b, (uint32_t)sizeof(FpBin), &sh.full[buf]);
 }
 
 __device__ __forceinline__ void cta_init(CtaShared &sh) {
@@ -599,61 +635,74 @@ __device__ __forceinline__ void cta_finish(CtaShared &sh) {
     }
 }
 
-// One work item (pass, observation tile) of one forest.  Bin bi of the item
-// goes through buffer bi % nbuf; the k-th copy ever issued into a buffer
-// completes its barrier's phase k, so a wait needs the buffer's copy count
-// at the item's start (use0) plus bi / nbuf.  Counting per buffer keeps the
-// phases right when items of forests with different nbuf share a CTA.  Every
-// warp waits for every bin's block, also for one it has no unit in: a warp
-// that ran ahead of a buffer's phases could not tell them apart.
-// HEADS: the forest has no super-nodes (walk_heads); its own build, since the
-// two walks in one kernel cost the other 8 % more instructions.
-template <int MODE, int DK, int HK, bool HEADS>
-__device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint8_t *smem, CtaShared &sh) {
-    constexpr bool D3 = DK >= 3;  // rows and thresholds are (remapped) order keys
-    constexpr bool LEAVES = MODE == FP_MODE_LEAVES, VALUES = MODE == FP_MODE_VALUES;
-    const int levels = HK >= 0 ? HK : p.levels;
-    const int R = p.R, F = p.F, C = p.C;
-    const int VR = LEAVES ? 0 : (VALUES ? 1 : C);  // counters per row: class votes, or one float sum
-    const uint32_t slab = p.slab;
-    const uint32_t hbuf0 = (uint32_t)(R >> 5) * slab;  // nbuf bin-block buffers, head_smem bytes each
-    const int nbuf = p.nbuf;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-    uint2 *ring = reinterpret_cast<uint2 *>(smem + hbuf0 + (uint32_t)(nbuf * p.head_smem)) + warp * FP_RING;
-    const unsigned lt_mask = (1u << lane) - 1u;
-
-    // one thread: stage bin b into a buffer
-    auto issue = [&](int b, int buf) {
-        sh.next[buf] = 0;
-        sh.done[buf] = 0;
-        sh.issued[buf] += 1;
-        stage_block_bulk(p, b, smem + hbuf0 + buf * p.head_smem, &sh.full[buf]);
-    };
-
-    // A CTA that gave up a wait skips its remaining items; each one records
-    // the timeout in its own forest's status, since its outputs stay unwritten
-    // (sh.abort is uniform here: it changes only inside the bin loop, and the
-    // previous item ended with a CTA barrier).
-    if (*(volatile int *)&sh.abort) {
-        if (tid == 0) report(p.status, FP_ERR_FLAG_TIMEOUT);
-        return;
+// Votes and classes of a tile whose splits were added up in p.acc (class 0:
+// the trees that voted for no other): a row's classes are spread over a group
+// of lanes, each reading its own (a thread per row reads them one after
+// another, an L2 latency for every few classes), and the maximum is found by
+// shuffles, lowest class on ties.  All threads of the CTA call this.
+__device__ __forceinline__ void finish_rows(const TravParams &p, int64_t row0, int rows) {
+    const int C = p.C;
+    int width = 1;  // lanes per row
+    while (width < C && width < 32) width *= 2;
+    const int lane = threadIdx.x & 31, sub = lane & (width - 1);
+    const int per_warp = 32 / width, per_cta = per_warp * (blockDim.x >> 5);
+    for (int i0 = 0; i0 < rows; i0 += per_cta) {
+        const int rr = i0 + (int)(threadIdx.x >> 5) * per_warp + lane / width;
+        const int64_t at = (row0 + rr) * C;
+        uint32_t bv = 0, others = 0;
+        int best = 0;
+        if (rr < rows) {
+            for (int c = sub; c < C; c += width) {
+                if (c == 0) continue;
+                const uint32_t x = __ldcg(p.acc + at + c);
+                others += x;
+                if (x > bv) { bv = x; best = c; }
+                if (p.out_votes && p.out_votes != p.acc) p.out_votes[at + c] = x;
+            }
+        }
+        for (int m = width >> 1; m > 0; m >>= 1) {
+            const uint32_t ov = __shfl_xor_sync(0xffffffffu, bv, m);
+            const int oc = __shfl_xor_sync(0xffffffffu, best, m);
+            others += __shfl_xor_sync(0xffffffffu, others, m);
+            if (ov > bv || (ov == bv && oc < best)) { bv = ov; best = oc; }
+        }
+        if (rr < rows && sub == 0) {
+            const uint32_t v0 = (uint32_t)p.T - others;
+            if (p.out_votes) p.out_votes[at] = v0;
+            if (p.out_class) p.out_class[row0 + rr] = v0 >= bv ? 0 : best;
+        }
     }
-    const int pass = (int)(item / p.n_tiles);
-    const int64_t tile = item - (int64_t)pass * p.n_tiles;
-    const int64_t row0 = tile * R;
-    const int rows = (int)(p.n - row0 < (int64_t)R ? p.n - row0 : (int64_t)R);
-    const int G = (rows + 31) >> 5;  // slabs in use
+}
 
-    // 1. rows -> shared memory, as order keys; 2. the first bins' blocks in flight
+// The start of an item: its bins and their first blocks in flight, its rows in
+// shared memory as order keys, its counters cleared.
+template <int MODE, int DK>
+__device__ __forceinline__ void begin_item(const TravParams &p, uint8_t *smem, CtaShared &sh, int64_t tile, int split,
+                                        uint32_t hbuf0) {
+    const int F = p.F, VR = MODE == FP_MODE_LEAVES ? 0 : (MODE == FP_MODE_VALUES ? 1 : p.C);
+    const uint32_t slab = p.slab;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5, nbuf = p.nbuf;
+    const int64_t row0 = tile * p.R;
+    const int rows = (int)(p.n - row0 < (int64_t)p.R ? p.n - row0 : (int64_t)p.R);
+    const int G = (rows + 31) >> 5;
     if (tid == 0) {
-        const FpPass ps = p.passes[pass];
-        sh.bin0 = ps.bin_begin;
-        sh.bin1 = ps.bin_end;
+        int b0 = 0, b1 = p.n_bins;
+        if (p.n_splits > 1 && p.n_splits == p.n_passes) {
+            const FpPass ps = p.passes[split];
+            b0 = ps.bin_begin;
+            b1 = ps.bin_end;
+        } else if (p.n_splits > 1) {
+            b0 = split * p.split_bins + min(split, p.split_more);
+            b1 = b0 + p.split_bins + (split < p.split_more ? 1 : 0);
+        }
+        sh.bin0 = b0;
+        sh.bin1 = b1;
         sh.tile = tile;
         uint32_t ph = 0;
         for (int i = 0; i < FP_NBUF; ++i) ph |= ((uint32_t)sh.issued[i] & 1u) << i;
         sh.phases = ph;
-        for (int i = 0; i < nbuf && ps.bin_begin + i < ps.bin_end; ++i) issue(ps.bin_begin + i, i);
+        for (int i = 0; i < nbuf && b0 + i < b1; ++i)
+            stage_bin(p, sh, b0 + i, p.bins[b0 + i], i, smem + hbuf0 + i * p.head_smem);
     }
     {
         // lane = row of a slab, 16 features at a time: loads along the row,
@@ -697,6 +746,118 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint
         const int g = u / VR;
         reinterpret_cast<uint32_t *>(smem + (uint32_t)g * slab)[(F + u - g * VR) * 32 + lane] = 0;
     }
+}
+
+// The end of an item, once every warp has finished its walks.
+template <int MODE>
+__device__ __forceinline__ void end_item(const TravParams &p, uint8_t *smem, CtaShared &sh) {
+    constexpr bool VALUES = MODE == FP_MODE_VALUES;
+    const int F = p.F, C = p.C, tid = threadIdx.x;
+    const uint32_t slab = p.slab;
+    const int64_t base = sh.tile * p.R;
+    const int nrows = (int)(p.n - base < (int64_t)p.R ? p.n - base : (int64_t)p.R);
+
+    // 5. the tile's results: from this CTA's shared memory, or, for a tile that
+    //    is cut into several splits, added up in global memory, where the CTA
+    //    that finishes the tile last completes it
+    const bool alone = p.n_splits == 1;
+    const bool go = !*(volatile int *)&sh.abort;
+    const uint32_t at0 = smem_u32(smem);
+    auto counter = [&](int rr, int c) {  // where a row's counter c lies
+        return at0 + (uint32_t)(rr >> 5) * slab + ((uint32_t)(F + c) << 7) + (uint32_t)(rr & 31) * 4u;
+    };
+    auto last_split = [&]() {  // true in the CTA that finishes the tile last
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) sh.last = atomicAdd(p.tile_done + sh.tile, 1u) == (unsigned)(p.n_splits - 1);
+        __syncthreads();
+        if (sh.last) __threadfence();
+        return sh.last != 0;
+    };
+    if (VALUES && go) {
+        if (alone) {
+            for (int rr = tid; rr < nrows; rr += blockDim.x)
+                p.out_val[base + rr] = p.vbias + p.vscale * __uint_as_float(lds(counter(rr, 0)));
+        } else {
+            float *dst = p.acc_val + base;
+            for (int rr = tid; rr < nrows; rr += blockDim.x) {
+                const float v = __uint_as_float(lds(counter(rr, 0)));
+                if (v != 0.0f) atomicAdd(dst + rr, v);
+            }
+            if (last_split())
+                for (int rr = tid; rr < nrows; rr += blockDim.x)
+                    p.out_val[base + rr] = p.vbias + p.vscale * __ldcg(dst + rr);
+        }
+    }
+    if (MODE == FP_MODE_VOTES && go) {
+        if (alone) {  // a thread per row; class 0 has the votes that no other class got
+            for (int rr = tid; rr < nrows; rr += blockDim.x) {
+                uint32_t *d = p.out_votes ? p.out_votes + (base + rr) * C : nullptr;
+                uint32_t rest = (uint32_t)p.T, bv = 0;
+                int best = 0;
+                for (int c = 1; c < C; ++c) {
+                    const uint32_t v = lds(counter(rr, c));
+                    rest -= v;
+                    if (v > bv) { bv = v; best = c; }
+                    if (d) d[c] = v;
+                }
+                if (d) d[0] = rest;
+                if (p.out_class) p.out_class[base + rr] = rest >= bv ? 0 : best;
+            }
+        } else {
+            // a warp per 32 rows and class: all of the CTA's warps have some,
+            // however few rows the tile has
+            const int groups = (nrows + 31) >> 5, lane = tid & 31;
+            for (int u = tid >> 5; u < groups * (C - 1); u += blockDim.x >> 5) {
+                const int c = u / groups + 1, rr = (u - (c - 1) * groups) * 32 + lane;
+                const uint32_t v = rr < nrows ? lds(counter(rr, c)) : 0u;
+                if (v) atomicAdd(p.acc + (base + rr) * C + c, v);
+            }
+            if (last_split()) finish_rows(p, base, nrows);
+        }
+    }
+}
+
+// One work item: one of the parts (splits) that the forest's bins are cut
+// into, and one observation tile.  The item's bins go through the buffers in
+// turn; the k-th copy ever issued into a buffer completes its barrier's phase
+// k, and every warp keeps the parities it waits for next (phases, from the
+// buffers' copy counts when the item starts).  Counting per buffer keeps the
+// phases right when items of forests with different nbuf share a CTA.  Every
+// warp waits for every bin's block, also for one it has no unit in: a warp
+// that ran ahead of a buffer's phases could not tell them apart.
+// HEADS: the forest has no super-nodes (walk_heads); its own build, since the
+// two walks in one kernel cost the other 8 % more instructions.
+template <int MODE, int DK, int HK, bool HEADS>
+__device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int split, uint8_t *smem,
+                                         CtaShared &sh) {
+    constexpr bool D3 = DK >= 3;  // rows and thresholds are (remapped) order keys
+    constexpr bool LEAVES = MODE == FP_MODE_LEAVES, VALUES = MODE == FP_MODE_VALUES;
+    const int levels = HK >= 0 ? HK : p.levels;
+    const int R = p.R;
+    const uint32_t slab = p.slab;
+    const uint32_t hbuf0 = (uint32_t)(R >> 5) * slab;  // nbuf bin-block buffers from here, head_smem bytes each
+    const int nbuf = p.nbuf;
+    const int tid = threadIdx.x, warp = tid >> 5, nwarps = blockDim.x >> 5;
+    const int lane = __shfl_sync(0xffffffffu, tid & 31, tid & 31);
+    // through a shuffle, which the compiler cannot redo in every step
+    const uint32_t base = __shfl_sync(0xffffffffu, smem_u32(smem), lane);
+    const uint32_t ring = base + hbuf0 + (uint32_t)(nbuf * p.head_smem + warp * FP_RING * 8);
+    const unsigned lt_mask = __shfl_sync(0xffffffffu, (1u << lane) - 1u, lane);
+
+    // A CTA that gave up a wait skips its remaining items; each one records
+    // the timeout in its own forest's status, since its outputs stay unwritten
+    // (sh.abort is uniform here: it changes only inside the bin loop, and the
+    // previous item ended with a CTA barrier).
+    if (*(volatile int *)&sh.abort) {
+        if (tid == 0) report(p.status, FP_ERR_FLAG_TIMEOUT);
+        return;
+    }
+    const int64_t row0 = tile * R;
+    const int rows = (int)(p.n - row0 < (int64_t)R ? p.n - row0 : (int64_t)R);
+    const int G = (rows + 31) >> 5;  // slabs in use
+
+    begin_item<MODE, DK>(p, smem, sh, tile, split, hbuf0);
     __syncthreads();
 
     LaneTask L;
@@ -705,11 +866,12 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint
     L.rt = 0;
     L.bad = 0;
     uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    Pending pend;
-    pend.on = false;
-    pend.at = 0;
-    pend.word = 0;
+    Pending pend, hpend;  // of the last deep step, of the last burst
+    pend.on = hpend.on = false;
+    pend.at = hpend.at = 0;
+    pend.word = hpend.word = 0;
     int head = 0, tail = 0;  // warp-uniform ring cursors
+    bool carried = false;    // the lanes' loads were issued in the bin before
 
     // unit u of a bin is slab u % G of its tree u / G: ceil(2^32 / G) divides by G
     const uint32_t inv_g = G > 1 ? 0xFFFFFFFFu / (uint32_t)G + 1u : 0u;
@@ -736,158 +898,101 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t item, uint
                 break;
             }
         }
-        const FpBin bn = p.bins[b];
+        const FpBin bn = sh.desc[buf];
         const int stride = bn.stride, nranks = bn.nranks, nexits = bn.nexits;
-        const uint32_t blk = hbuf0 + (uint32_t)(buf * p.head_smem);
+        const uint32_t blk = base + hbuf0 + (uint32_t)(buf * p.head_smem);
         const uint32_t exits = blk + (uint32_t)(nranks * stride * (levels == 2 ? 16 : 8));
 
-        if (HEADS) walk_heads<MODE, D3, HK>(p, smem, sh, bn, blk, exits, buf, rows, G, inv_g, L.bad);
+        if (HEADS) walk_heads<MODE, D3, HK>(p, base, sh, bn, blk, exits, buf, rows, G, inv_g, L.bad);
         const int units = bn.width * G;
-        while (!HEADS) {
-            ld_super(p.deep, L.ref, w);  // in flight during the burst below
-            settle<MODE>(p, smem, sh, pend);
-            if (tail - head <= p.refill) {
-                // burst: the unit's 32 rows through the head of its tree, all lanes together
+        if (!HEADS) {
+            for (;;) {
+                // deep steps until the ring runs low
+                if (!carried) ld_super(p.deep, L.ref, w);
+                carried = false;
+                settle<MODE>(p, sh, pend);
+                settle<MODE>(p, sh, hpend);
+                while (__any_sync(0xffffffffu, tail - head > p.refill)) {
+                    deep_finish<MODE, DK>(p, L, pend, w);
+                    pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
+                    ld_super(p.deep, L.ref, w);
+                    settle<MODE>(p, sh, pend);
+                }
                 int unit = 0;
                 if (lane == 0) unit = atomicAdd(&sh.next[buf], 1);
                 unit = __shfl_sync(0xffffffffu, unit, 0);
-                if (unit >= units) {  // all taken: use the load in flight, then move on
-                    if (__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) deep_finish<MODE, DK>(p, smem, L, pend, w);
-                    pop_tasks<MODE>(p, ring, head, tail, L, lt_mask);
-                    break;
-                }
+                if (__any_sync(0xffffffffu, unit >= units)) break;  // all taken
                 const int uk = G > 1 ? (int)__umulhi((uint32_t)unit, inv_g) : unit, ug = unit - uk * G;
-                const uint32_t xb = (uint32_t)ug * slab + (uint32_t)lane * 4u;
+                const uint32_t xb = base + (uint32_t)ug * slab + (uint32_t)lane * 4u;
                 const int r2 = ug * 32 + lane;
                 const bool my = r2 < rows;
                 const uint32_t at =
-                    head_walk<D3, HK>(p, smem, blk, exits, uk, stride, nranks, nexits, xb, my);
+                    head_walk<D3, HK>(p, blk, exits, uk, stride, nranks, nexits, xb, my);
                 const bool ok = HK > 0 || at != FP_NO_EXIT;
-                const uint32_t er = ok ? lds(smem, at) : FP_NO_CLASS;
+                const uint32_t er = ok ? lds(at) : FP_NO_CLASS;
                 const bool push = my && !(er & FP_REF_LEAF);
                 if (my && !push) {  // a leaf in the head, or right below it
                     const uint32_t cls = er & 0x7FFFFFFFu;
                     if (LEAVES) {
                         L.bad |= !ok;
-                        if (ok)
-                            put_leaf(p, sh, (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11),
-                                     p.pheads[(bn.phead_off >> 2) + ((at - exits) >> 2)]);
+                        hpend.on = ok;
+                        hpend.at = (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11);
+                        if (ok) hpend.word = (uint32_t)__ldg(p.pheads + (bn.phead_off >> 2) + ((at - exits) >> 2));
                     } else if (VALUES) {
                         L.bad |= cls >= p.n_vals;
-                        if (cls < p.n_vals) add_value(p, smem, xb, __ldg(p.leaf_val + cls));
+                        hpend.on = cls < p.n_vals;
+                        hpend.at = xb;
+                        if (hpend.on) hpend.word = __float_as_uint(__ldg(p.leaf_val + cls));
                     } else {
-                        L.bad |= !vote(p, smem, true, xb, cls);
+                        L.bad |= !vote(p, true, xb, cls);
                     }
                 }
                 const unsigned pm = __ballot_sync(0xffffffffu, push);
                 if (push)
-                    ring[(tail + __popc(pm & lt_mask)) & (FP_RING - 1)] =
-                        make_uint2(er, LEAVES ? (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11) : xb);
+                    sts64(ring + (uint32_t)((tail + __popc(pm & lt_mask)) & (FP_RING - 1)) * 8u, er,
+                          LEAVES ? (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11) : xb);
                 tail += __popc(pm);
                 __syncwarp();
+                deep_finish<MODE, DK>(p, L, pend, w);
+                pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
             }
-            if (__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) deep_finish<MODE, DK>(p, smem, L, pend, w);
-            pop_tasks<MODE>(p, ring, head, tail, L, lt_mask);
         }
         // this warp reads the bin's block no more; the last warp refills the buffer
         __syncwarp();
         if (lane == 0) {
             const int done = atomicAdd(&sh.done[buf], 1);
-            if (done == nwarps - 1 && b + nbuf < sh.bin1 && !*(volatile int *)&sh.abort) issue(b + nbuf, buf);
+            if (done == nwarps - 1 && b + nbuf < sh.bin1 && !*(volatile int *)&sh.abort) {
+                const FpBin next = p.bins[b + nbuf];
+                stage_bin(p, sh, b + nbuf, next, buf, smem + hbuf0 + buf * p.head_smem);
+            }
+        }
+        __syncwarp();
+        // the load in flight is used here, or, where a bin has fewer units than
+        // there are warps, carried into the next bin: waiting for it in every
+        // bin would cost most warps an L2 latency for nothing
+        carried = units < nwarps;
+        if (!HEADS && !carried && __any_sync(0xffffffffu, L.ref != FP_NO_TASK)) {
+            deep_finish<MODE, DK>(p, L, pend, w);
+            pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
         }
         if (++buf == nbuf) buf = 0;
-        __syncwarp();
     }
     const bool aborted = *(volatile int *)&sh.abort != 0;
     // drain: the item's last pending and running tasks
     for (; !HEADS && !aborted;) {
         __syncwarp();
-        pop_tasks<MODE>(p, ring, head, tail, L, lt_mask);
+        pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
         if (!__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) break;
         ld_super(p.deep, L.ref, w);
-        settle<MODE>(p, smem, sh, pend);
-        deep_finish<MODE, DK>(p, smem, L, pend, w);
+        settle<MODE>(p, sh, pend);
+        deep_finish<MODE, DK>(p, L, pend, w);
     }
-    settle<MODE>(p, smem, sh, pend);
+    settle<MODE>(p, sh, pend);
+    settle<MODE>(p, sh, hpend);
     if (L.bad) report(p.status, FP_ERR_FLAG_DEVICE);
     __syncthreads();
 
-    // what the walk did not keep in registers
-    const int64_t base = sh.tile * p.R;
-    const int nrows = (int)(p.n - base < (int64_t)p.R ? p.n - base : (int64_t)p.R);
-
-    // 5. values: bias + scale * the row's sum (several passes: summed in global
-    //    memory, the CTA finishing a tile's last pass writes the result)
-    if (VALUES && !*(volatile int *)&sh.abort) {
-        auto sum_of = [&](int rr) {
-            return __uint_as_float(lds(smem, (uint32_t)(rr >> 5) * slab + ((uint32_t)F << 7) + (uint32_t)(rr & 31) * 4u));
-        };
-        if (p.n_passes == 1) {
-            for (int rr = tid; rr < nrows; rr += blockDim.x) p.out_val[base + rr] = p.vbias + p.vscale * sum_of(rr);
-        } else {
-            float *dst = p.acc_val + base;
-            for (int rr = tid; rr < nrows; rr += blockDim.x) {
-                const float v = sum_of(rr);
-                if (v != 0.0f) atomicAdd(dst + rr, v);
-            }
-            __threadfence();
-            __syncthreads();
-            if (tid == 0) sh.last = atomicAdd(p.tile_done + sh.tile, 1u) == (unsigned)(p.n_passes - 1);
-            __syncthreads();
-            if (sh.last) {
-                __threadfence();
-                for (int rr = tid; rr < nrows; rr += blockDim.x)
-                    p.out_val[base + rr] = p.vbias + p.vscale * __ldcg(dst + rr);
-            }
-        }
-    }
-    // 5. votes and class: a thread per row; class 0 has the votes that no other class got
-    if (MODE == FP_MODE_VOTES && !*(volatile int *)&sh.abort) {
-        const FpBin first = p.bins[sh.bin0], last = p.bins[sh.bin1 - 1];
-        const uint32_t trees = (uint32_t)(last.first_tree + last.width - first.first_tree);
-        uint32_t *const dst = p.n_passes == 1 ? p.out_votes : p.acc;
-        for (int rr = tid; rr < nrows; rr += blockDim.x) {
-            const uint32_t vb = (uint32_t)(rr >> 5) * slab + ((uint32_t)F << 7) + (uint32_t)(rr & 31) * 4u;
-            uint32_t *d = dst ? dst + (base + rr) * C : nullptr;
-            uint32_t rest = trees, bv = 0;
-            int best = 0;
-            for (int c = 1; c < C; ++c) {
-                const uint32_t v = lds(smem, vb + (uint32_t)c * 128u);
-                rest -= v;
-                if (v > bv) { bv = v; best = c; }
-                if (p.n_passes == 1) {
-                    if (d) d[c] = v;
-                } else if (v) {
-                    atomicAdd(d + c, v);
-                }
-            }
-            if (p.n_passes == 1) {
-                if (d) d[0] = rest;
-                if (p.out_class) p.out_class[base + rr] = rest >= bv ? 0 : best;
-            } else if (rest) {
-                atomicAdd(d, rest);
-            }
-        }
-        if (p.n_passes > 1 && p.out_class) {
-            __threadfence();
-            __syncthreads();
-            if (tid == 0) sh.last = atomicAdd(p.tile_done + sh.tile, 1u) == (unsigned)(p.n_passes - 1);
-            __syncthreads();
-            if (sh.last) {
-                __threadfence();
-                for (int rr = tid; rr < nrows; rr += blockDim.x) {
-                    const uint32_t *v = p.acc + (base + rr) * C;
-                    int best = 0;
-                    uint32_t bv = __ldcg(v);
-                    for (int c = 1; c < C; ++c) {
-                        const uint32_t x = __ldcg(v + c);
-                        if (x > bv) { bv = x; best = c; }
-                    }
-                    p.out_class[base + rr] = best;
-                }
-            }
-        }
-    }
+    end_item<MODE>(p, smem, sh);
     __syncthreads();  // the next item reuses shared memory
 }
 
@@ -910,18 +1015,27 @@ __global__ void fp_inline_values_kernel(uint8_t *heads, const FpBin *bins, const
 // two 24-warp or three 16-warp CTAs share an SM when shared memory allows:
 // more warps to hide the latency of the dependent loads of each walk.
 template <int MODE, int MINB, int DK, int HK, bool HEADS>
-__global__ void __launch_bounds__(MINB == 1 ? 1024 : 768, MINB) fp_traverse_kernel(const TravParams p) {
+__global__ void __launch_bounds__(MINB == 1 ? 1024 : 768, MINB) fp_traverse_kernel(const __grid_constant__ TravParams p) {
     extern __shared__ __align__(16) uint8_t smem[];
     __shared__ CtaShared sh;
     cta_init(sh);
-    for (int64_t item = blockIdx.x; item < p.n_items; item += gridDim.x) 
-        run_item<MODE, DK, HK, HEADS>(p, item, smem, sh);
+    // all tiles of a split, then the next one's, so that the CTAs walk the same
+    // bins at a time
+    int64_t tile = blockIdx.x;
+    int split = 0;
+    for (;;) {
+        for (; tile >= p.n_tiles && split < p.n_splits; tile -= p.n_tiles) ++split;
+        if (split >= p.n_splits) break;
+        run_item<MODE, DK, HK, HEADS>(p, tile, split, smem, sh);
+        tile += gridDim.x;
+    }
     cta_finish(sh);
 }
 
 // Several forests and batches in one persistent launch: the work items of
-// all batches form one list (batch by batch, pass-major within a batch),
-// handed out to CTAs through a global counter so uneven batches balance.
+// all batches form one list (batch by batch, split by split within a batch),
+// handed out to CTAs through a global counter so uneven batches balance; how
+// long items are is chosen for the launch (fp_device.cu).
 #define FP_MAX_BATCH 32
 
 struct BatchParams {
@@ -948,12 +1062,15 @@ __global__ void __launch_bounds__(1024, 1) fp_traverse_batched_kernel(const __gr
         if (item >= total) break;
         int j = 0;
         while (j + 1 < bp.k && bp.item_begin[j + 1] <= item) ++j;
+        const int64_t own = item - bp.item_begin[j];
+        const int split = (int)(own / bp.p[j].n_tiles);
+        const int64_t tile = own - split * bp.p[j].n_tiles;
         if (KIND == 3 || (KIND == 0 && bp.p[j].deep_kind == 3))
-            run_item<FP_MODE_VOTES, 3, HK, false>(bp.p[j], item - bp.item_begin[j], smem, sh);
+            run_item<FP_MODE_VOTES, 3, HK, false>(bp.p[j], tile, split, smem, sh);
         else if (KIND == 4 || (KIND == 0 && bp.p[j].deep_kind == 4))
-            run_item<FP_MODE_VOTES, 4, HK, false>(bp.p[j], item - bp.item_begin[j], smem, sh);
+            run_item<FP_MODE_VOTES, 4, HK, false>(bp.p[j], tile, split, smem, sh);
         else
-            run_item<FP_MODE_VOTES, 2, HK, false>(bp.p[j], item - bp.item_begin[j], smem, sh);
+            run_item<FP_MODE_VOTES, 2, HK, false>(bp.p[j], tile, split, smem, sh);
     }
     cta_finish(sh);
 }
