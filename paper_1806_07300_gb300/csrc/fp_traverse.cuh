@@ -536,22 +536,61 @@ __device__ __forceinline__ uint32_t head_walk(const TravParams &p, uint32_t blk,
     return e < (uint32_t)nexits ? exits + 4u * (e * (uint32_t)stride + (uint32_t)k) : FP_NO_EXIT;
 }
 
+// The walks of one row through the paired heads of N neighbouring tree columns
+// at once, each as in head_walk: the N trees' loads are in flight together.
+template <bool KEYS, int N>
+__device__ __forceinline__ void head_walks(const TravParams &p, uint32_t blk, uint32_t exits, int k, int stride,
+                                           uint32_t xb, uint32_t exit_at[N]) {
+    const uint32_t rec = (uint32_t)stride * 16u, at0 = blk + (uint32_t)k * 16u;
+    const uint32_t left = rec - 3u * at0, right = left + 2u * rec;
+    uint32_t at[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) at[i] = at0 + 16u * i;
+#pragma unroll 1
+    for (int l = 0; l <= p.depth; l += 2) {
+        uint4 nd[N];
+        uint32_t x[N];
+        bool r0[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) nd[i] = lds128(at[i]);
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] = lds(xb + ((nd[i].w & 1023u) << 7));
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            r0[i] = !goes_left<KEYS>(x[i], nd[i].x);
+            x[i] = lds(xb + ((nd[i].w >> (r0[i] ? 20 - 7 : 10 - 7)) & (1023u << 7)));
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const bool r1 = !goes_left<KEYS>(x[i], r0[i] ? nd[i].z : nd[i].y);
+            at[i] = 4u * at[i] + (r0[i] ? right : left) + (r1 ? rec : 0u) - 48u * i;  // column k + i begins 16 i later
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) exit_at[i] = exits + ((at[i] - exits) >> 2);
+}
+
 // Forests whose trees end in the interleaved heads (no super-nodes: shallow
 // trees, such as boosted ones).  Every walk of a slab through a tree ends
 // together, so nothing is pushed or popped: a warp takes a slab and a run of
-// up to 8 of the bin's trees, keeps the row's sum of leaf values (or its votes
+// up to 32 of the bin's trees, keeps the row's sum of leaf values (or its votes
 // for class 1 of 2) in a register over the run, and adds it to the slab's
 // counter once.  A task costs the head walk, one exit word and one add; as a
 // burst of its own it also paid for the claim, its division, the read of its
-// value from global memory and an atomic (256 boosted trees of six levels, 2 M
-// rows: 2.93 ms as bursts, 1.53 ms as runs; bound by instruction issue).
+// value from global memory and an atomic.  FP_HEAD_TREES trees are walked at a
+// time, since one tree's walk is a chain of shared-memory latencies.  256
+// boosted trees of six levels, 2 M rows: 2.93 ms as bursts, 1.47 ms one tree at
+// a time, 1.21, 1.19, 1.15 and 1.22 ms with 2, 3, 4 and 6 at a time (runs of
+// 16; 1.145 ms with 4 in runs of 32); bound by instruction issue.
+#define FP_HEAD_TREES 4
+
 template <int MODE, bool KEYS, int HK>
 __device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, CtaShared &sh, const FpBin &bn,
                                            uint32_t blk, uint32_t exits, int buf, int rows, int G, uint32_t inv_g,
                                            int &bad) {
     const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    // runs of 8 trees, shorter when the bin would leave warps without one
-    const int run = max(1, min(8, bn.width * G / nwarps));
+    // runs of 32 trees, shorter when the bin would leave warps without one
+    const int run = max(1, min(32, bn.width * G / nwarps));
     const int units = (bn.width + run - 1) / run * G;
     for (;;) {
         int unit = 0;
@@ -565,12 +604,7 @@ __device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, C
         const int k1 = min(bn.width, (c + 1) * run);
         float sum = 0.0f;
         uint32_t ones = 0;
-        for (int k = c * run; k < k1; ++k) {
-            const uint32_t at = head_walk<KEYS, HK>(p, blk, exits, k, bn.stride, bn.nranks, bn.nexits, xb, my);
-            if (HK <= 0 && at == FP_NO_EXIT) {
-                bad |= my;
-                continue;
-            }
+        auto take = [&](int k, uint32_t at) {  // the row's walk through tree k ended on the exit word `at`
             if (MODE == FP_MODE_VALUES) {
                 sum += __uint_as_float(lds(at));  // the exits hold the leaves' values themselves
             } else if (MODE == FP_MODE_LEAVES) {
@@ -586,6 +620,23 @@ __device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, C
                     bad |= !vote(p, my, xb, cls);
                 }
             }
+        };
+        int k = c * run;
+        if (HK == 2) {
+            for (; k + FP_HEAD_TREES <= k1; k += FP_HEAD_TREES) {
+                uint32_t at[FP_HEAD_TREES];
+                head_walks<KEYS, FP_HEAD_TREES>(p, blk, exits, k, bn.stride, xb, at);
+#pragma unroll
+                for (int i = 0; i < FP_HEAD_TREES; ++i) take(k + i, at[i]);
+            }
+        }
+        for (; k < k1; ++k) {
+            const uint32_t at = head_walk<KEYS, HK>(p, blk, exits, k, bn.stride, bn.nranks, bn.nexits, xb, my);
+            if (HK <= 0 && at == FP_NO_EXIT) {
+                bad |= my;
+                continue;
+            }
+            take(k, at);
         }
         if (MODE == FP_MODE_VALUES && my) add_value(p, xb, sum);
         if (MODE == FP_MODE_VOTES && my && p.C == 2 && ones)
