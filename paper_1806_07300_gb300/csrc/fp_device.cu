@@ -27,11 +27,16 @@ struct fp_device_forest {
     std::vector<FpBin> bins;
     std::vector<FpPass> passes;
     uint8_t *d_image = nullptr;
+    uint8_t *d_compact = nullptr;  // one-word level heads, after their bins (NULL: none)
+    int64_t compact_bins_bytes = 0;
     int32_t *d_status = nullptr;
     int32_t R = 0;            // observation tile actually launched (fits shared memory)
     int32_t threads = 0;
     int32_t refill = 8;
-    int32_t head_smem = 0;
+    int32_t levels = 0;       // head kind of a launch of this forest alone (TravParams::levels)
+    int32_t head_smem = 0;    // bytes of one of its bin-block buffers ...
+    int32_t head_plan = 0;    // ... of one with the packed blocks, which tiles are fitted beside ...
+    int32_t head_shared = 0;  // ... and of one in a launch with other forests
     int32_t nbuf = 3;                          // bin-block buffers
     size_t smem_votes = 0, smem_leaves = 0, smem_values = 0;
     int32_t grid_votes = 0, grid_leaves = 0, grid_values = 0;  // resident CTAs for a persistent launch
@@ -98,16 +103,24 @@ size_t smem_bytes(int R, int F, int head_smem, int nbuf, int C, int warps, bool 
 // for several CTAs per SM (<= 42 registers), larger blocks the one-CTA build ...
 template <int MODE, int DK, int HK>
 void (*traverse_kernel_sized(const fp_device_forest *f))(TravParams) {
-    if (f->hdr.n_super == 0) return fp_traverse_kernel<MODE, 1, DK, HK, true>;  // one build serves every CTA size
     return f->threads <= 768 ? fp_traverse_kernel<MODE, 2, DK, HK, false> : fp_traverse_kernel<MODE, 1, DK, HK, false>;
 }
 
-// ... and its head kind (compiled in: 0 ranked, 1 level slots, 2 paired).
+// ... and its head kind (compiled in: 0 ranked, 1 level slots, 2 paired, 3
+// level slots of one word).
 template <int MODE, int DK>
 void (*traverse_kernel_deep(const fp_device_forest *f))(TravParams) {
-    switch (f->hdr.head_select) {
-        case 1: return traverse_kernel_sized<MODE, DK, 1>(f);
+    if (f->hdr.n_super == 0) {  // one build serves every CTA size
+        switch (f->levels) {
+            case 1: return fp_traverse_kernel<MODE, 1, DK, 1, true>;
+            case 2: return fp_traverse_kernel<MODE, 1, DK, 2, true>;
+            default: return fp_traverse_kernel<MODE, 1, DK, 0, true>;
+        }
+    }
+    switch (f->levels) {  // unpaired level slots have float thresholds only, those of one word have keys only
+        case 1: return traverse_kernel_sized<MODE, DK, DK == 2 ? 1 : 0>(f);
         case 2: return traverse_kernel_sized<MODE, DK, 2>(f);
+        case 3: return traverse_kernel_sized<MODE, DK, DK == 2 ? 0 : 3>(f);
         default: return traverse_kernel_sized<MODE, DK, 0>(f);
     }
 }
@@ -125,13 +138,14 @@ void (*traverse_kernel(const fp_device_forest *f))(TravParams) {
 }
 
 // Every instance of the batched kernel: super-node kind (0 mixed, 2, 3, 4) x
-// head kind (-1 mixed, 0 ranked, 1, 2).
+// head kind (-1 mixed, 0 ranked, 1, 2, 3).
 template <int KIND>
 void add_batched(std::vector<void (*)(BatchParams)> &v) {
     v.push_back(fp_traverse_batched_kernel<KIND, -1>);
     v.push_back(fp_traverse_batched_kernel<KIND, 0>);
     v.push_back(fp_traverse_batched_kernel<KIND, 1>);
     v.push_back(fp_traverse_batched_kernel<KIND, 2>);
+    v.push_back(fp_traverse_batched_kernel<KIND, 3>);
 }
 
 const std::vector<void (*)(BatchParams)> &batched_kernels() {
@@ -146,10 +160,10 @@ const std::vector<void (*)(BatchParams)> &batched_kernels() {
     return v;
 }
 
-// The instance for a launch: index 4 * kind + (head kind + 1) into batched_kernels().
+// The instance for a launch: index 5 * kind + (head kind + 1) into batched_kernels().
 void (*batched_kernel(int kind, int hk))(BatchParams) {
     const int ki = kind >= 2 ? kind - 1 : 0;  // 0 mixed, 1 two levels, 2 format 1, 3 format 2
-    return batched_kernels()[(size_t)(4 * ki + (hk + 1))];
+    return batched_kernels()[(size_t)(5 * ki + (hk + 1))];
 }
 
 // The dynamic shared-memory limit is an attribute of the kernel instance,
@@ -191,10 +205,10 @@ int launch_setup(fp_device_forest *f, int32_t tile, int32_t warps, int32_t refil
     const size_t budget = (size_t)max_optin - 256;  // leaves room for the static shared variables
     const int C = f->hdr.n_classes, F = f->hdr.n_features;
     int R = tile;
-    while (R > 32 && smem_bytes(R, F, f->head_smem, nbuf, C, warps, false) > budget) R -= 32;
-    if (smem_bytes(R, F, f->head_smem, nbuf, C, warps, false) > budget) {
+    while (R > 32 && smem_bytes(R, F, f->head_plan, nbuf, C, warps, false) > budget) R -= 32;
+    if (smem_bytes(R, F, f->head_plan, nbuf, C, warps, false) > budget) {
         fp_set_error("a 32-row tile, the bin-block buffers and the task rings need %zu bytes of shared memory (limit %zu)",
-                     smem_bytes(R, F, f->head_smem, nbuf, C, warps, false), budget);
+                     smem_bytes(R, F, f->head_plan, nbuf, C, warps, false), budget);
         return FP_EUNSUPPORTED;
     }
     fp_device_forest g = *f;
@@ -367,7 +381,8 @@ int plan_rows(const fp_device_forest *f, int64_t n, int32_t grid, bool split, bo
     return 2;
 }
 
-TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
+// levels: the head kind that the launch walks this forest with.
+TravParams base_params(const fp_device_forest *f, const float *X, int64_t n, int32_t levels) {
     TravParams p;
     memset(&p, 0, sizeof p);
     const FpImageHeader &h = f->hdr;
@@ -390,9 +405,16 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n) {
     p.n_passes = h.n_passes;
     p.n_bins = h.n_bins;
     p.split_bins = h.n_bins;
-    p.head_smem = f->head_smem;
+    p.head_smem = levels == f->levels ? f->head_smem : f->head_shared;
     p.nbuf = f->nbuf;
-    p.levels = h.head_select == 3 ? 0 : h.head_select;  // kernel: 0 ranked, 1 level slots, 2 paired
+    p.levels = levels;
+    if (levels == 3) {
+        p.packed_kind = h.head_select;
+        p.packed_heads = p.heads;
+        p.packed_bins = p.bins;
+        p.bins = reinterpret_cast<const FpBin *>(f->d_compact);
+        p.heads = f->d_compact + f->compact_bins_bytes;
+    }
     p.leaf_val = reinterpret_cast<const float *>(f->d_image + h.off_values);
     p.n_vals = (uint32_t)h.n_values;
     p.depth = h.depth;
@@ -470,6 +492,51 @@ int check_device(const fp_device_forest *f) {
 
 }  // namespace
 
+// The one-word level heads of an uploaded forest (fp_compact_heads_kernel) and
+// their bins; the forest then walks those.  Waits for the stream.
+static int compact_heads(fp_device_forest *f, cudaStream_t s) {
+    const FpImageHeader &h = f->hdr;
+    std::vector<FpBin> bins;
+    try {
+        bins = f->bins;
+    } catch (const std::bad_alloc &) {
+        fp_set_error("fp_upload: out of host memory");
+        return FP_ENOMEM;
+    }
+    const int32_t nodes = (1 << (h.depth + 1)) - 1;
+    int64_t off = 0;
+    int32_t largest = 0;
+    for (FpBin &b : bins) {
+        b.nranks = nodes;
+        b.head_bytes = (uint32_t)(((int64_t)(nodes + b.nexits) * b.stride * 4 + 15) & ~(int64_t)15);
+        b.head_off = (uint32_t)off;  // below the packed block's, which fits
+        off += b.head_bytes;
+        largest = std::max<int32_t>(largest, (int32_t)b.head_bytes);
+    }
+    f->compact_bins_bytes = ((int64_t)(bins.size() * sizeof(FpBin)) + 255) & ~(int64_t)255;
+    cudaError_t e = cudaMalloc(&f->d_compact, (size_t)(f->compact_bins_bytes + off));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(heads)");
+    e = cudaMemcpyAsync(f->d_compact, bins.data(), bins.size() * sizeof(FpBin), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(heads)");
+    fp_compact_heads_kernel<<<(unsigned)bins.size(), 256, 0, s>>>(
+        f->d_compact + f->compact_bins_bytes, reinterpret_cast<const FpBin *>(f->d_compact),
+        f->d_image + h.off_heads, reinterpret_cast<const FpBin *>(f->d_image + h.off_bins), h.head_select,
+        (1u << h.feature_bits) - 1u);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // before the host's bins go
+    if (e != cudaSuccess) return cuda_fail(e, "fp_compact_heads_kernel");
+    f->head_shared = largest;
+    // Alone, paired heads of at most four levels are walked as packed: their
+    // records are few enough for a warp to read most of them without bank
+    // conflicts (784-feature rows, heads 0..3, 250,000 rows: 1482 us, 1494 us
+    // with one-word slots).
+    if (f->levels == 1 || h.depth > 3) {
+        f->levels = 3;
+        f->head_smem = largest;
+    }
+    return FP_OK;
+}
+
 extern "C" int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_forest **out) {
     if (!out || !pf) {
         fp_set_error("fp_upload: NULL argument");
@@ -511,13 +578,19 @@ extern "C" int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_for
     }
     e = cudaStreamSynchronize(s);  // the caller may free the host image on return
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaStreamSynchronize"); goto fail; }
-    f->head_smem = (h->max_head_bytes + 15) & ~15;
+    f->head_smem = f->head_plan = f->head_shared = (h->max_head_bytes + 15) & ~15;
+    f->levels = h->head_select == 3 ? 0 : h->head_select;
     fit_costs(f);
+    if (h->n_super > 0 && deep_kind(*h) >= 3 && f->levels != 0) {
+        rc = compact_heads(f, s);
+        if (rc) goto fail;
+    }
     rc = launch_setup(f, h->obs_tile, h->warps_per_cta, h->refill_lanes, h->bin_buffers);
     if (rc) goto fail;
     *out = f;
     return FP_OK;
 fail:
+    if (f->d_compact) cudaFree(f->d_compact);
     if (f->d_image) cudaFree(f->d_image);
     if (f->d_status) cudaFree(f->d_status);
     delete f;
@@ -570,7 +643,7 @@ int predict_votes(const fp_device_forest *f, const float *X, int64_t n, uint32_t
             if (rc && h.n_passes > 1 && !whole) return rc;
             if (rc) pt.shape.S = 1;  // the same rows without scratch
         }
-        TravParams p = base_params(f, X + pt.row0 * h.n_features, pt.n);
+        TravParams p = base_params(f, X + pt.row0 * h.n_features, pt.n, f->levels);
         set_shape(p, pt.shape);
         p.out_votes = votes;
         p.out_class = out_class ? out_class + pt.row0 : nullptr;
@@ -638,7 +711,7 @@ extern "C" int fp_predict_values(const fp_device_forest *f, const float *X, int6
             if (rc && h.n_passes > 1) return rc;
             if (rc) pt.shape.S = 1;  // the same rows without scratch
         }
-        TravParams p = base_params(f, X + pt.row0 * h.n_features, pt.n);
+        TravParams p = base_params(f, X + pt.row0 * h.n_features, pt.n, f->levels);
         set_shape(p, pt.shape);
         p.slab = (uint32_t)slab_bytes(h.n_features, 1, false);
         p.vscale = scale;
@@ -744,7 +817,7 @@ extern "C" int fp_predict_leaves(const fp_device_forest *f, const float *X, int6
     const int k = plan_rows(f, n, f->grid_leaves, false, true, parts);
     for (int i = 0; i < k; ++i) {
         const Part &pt = parts[i];
-        TravParams p = base_params(f, X + pt.row0 * f->hdr.n_features, pt.n);
+        TravParams p = base_params(f, X + pt.row0 * f->hdr.n_features, pt.n, f->levels);
         set_shape(p, pt.shape);
         p.slab = (uint32_t)slab_bytes(f->hdr.n_features, 0, true);
         p.out_leaf = out_leaf + pt.row0 * f->hdr.n_trees;
@@ -814,6 +887,7 @@ extern "C" void fp_release(fp_device_forest *f) {
     cudaGetDevice(&prev);
     if (prev != f->device) cudaSetDevice(f->device);
     cudaDeviceSynchronize();
+    cudaFree(f->d_compact);
     cudaFree(f->d_image);
     cudaFree(f->d_status);
     if (prev >= 0 && prev != f->device) cudaSetDevice(prev);
@@ -879,9 +953,9 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
         if (bt.n == 0 || (!bt.out_votes && !bt.out_class)) continue;
         const FpImageHeader &h = f->hdr;
         int R = f->R;
-        while (R > 32 && smem_bytes(R, h.n_features, f->head_smem, f->nbuf, h.n_classes, warps, false) > budget) R -= 32;
-        const size_t need = smem_bytes(R, h.n_features, f->head_smem, f->nbuf, h.n_classes, warps, false);
-        if (need > budget) {
+        while (R > 32 && smem_bytes(R, h.n_features, f->head_plan, f->nbuf, h.n_classes, warps, false) > budget) R -= 32;
+        const size_t need = smem_bytes(R, h.n_features, f->head_shared, f->nbuf, h.n_classes, warps, false);
+        if (smem_bytes(R, h.n_features, f->head_plan, f->nbuf, h.n_classes, warps, false) > budget) {
             fp_set_error("fp_predict_batched: batch %d does not fit shared memory with %d warps", j, warps);
             return FP_EUNSUPPORTED;
         }
@@ -913,7 +987,9 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
     for (int32_t i = 0; i < m; ++i) {
         const fp_device_forest *f = forests[live[i]];
         const fp_batch &bt = batches[live[i]];
-        TravParams p = base_params(f, bt.X, bt.n);
+        // one-word heads for every forest that has them, so that most launches
+        // need one kind of walk (mixed kinds: 4 % longer)
+        TravParams p = base_params(f, bt.X, bt.n, f->d_compact ? 3 : f->levels);
         set_shape(p, shape_within(f, bt.n, max_R[i], most));
         p.out_votes = bt.out_votes;
         p.out_class = bt.out_class;
