@@ -209,6 +209,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 // CTA-wide state shared by the items a CTA runs.
 struct __align__(16) CtaShared {
     FpBin desc[FP_NBUF];      // the record of each buffer's bin
+    uint4 ahead[FP_NBUF];     // the first half of the record of the bin that refills the buffer
     uint64_t full[FP_NBUF];   // block staged (bulk copy done)
     int next[FP_NBUF];        // next untaken unit of the buffer's bin
     int done[FP_NBUF];        // warps done with the buffer's bin
@@ -698,21 +699,24 @@ __device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, C
     }
 }
 
-// One thread: copy bin b's block (its record: bn) into a buffer with the
-// bulk-copy engine, and its record beside it, so that the warps that walk the
-// bin do not wait for that from global memory once more.
-__device__ __forceinline__ void stage_bin(const TravParams &p, CtaShared &sh, int b, const FpBin &bn, int buf,
-                                          uint8_t *dst) {
+// One thread: copy bin b's block into a buffer with the bulk-copy engine, its
+// record beside it, and half the record of the bin that will follow it there,
+// so that neither the warps that walk the bin nor the thread that refills the
+// buffer wait for one from global memory.
+__device__ __forceinline__ void stage_bin(const TravParams &p, CtaShared &sh, int b, uint32_t head_off,
+                                          uint32_t head_bytes, int buf, uint8_t *dst) {
+    const bool more = b + p.nbuf < p.n_bins;
     sh.next[buf] = 0;
     sh.done[buf] = 0;
     sh.issued[buf] += 1;
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // earlier reads of dst come first
     asm volatile("mbarrier.arrive.expect_tx.release.cta.shared::cta.b64 _, [%0], %1;\n" ::"r"(
                      smem_u32(&sh.full[buf])),
-                 "r"(bn.head_bytes + (uint32_t)sizeof(FpBin))
+                 "r"(head_bytes + (uint32_t)sizeof(FpBin) + (more ? 16u : 0u))
                  : "memory");
-    bulk_copy(dst, p.heads + bn.head_off, bn.head_bytes, &sh.full[buf]);
+    bulk_copy(dst, p.heads + head_off, head_bytes, &sh.full[buf]);
     bulk_copy(&sh.desc[buf], p.bins + b, (uint32_t)sizeof(FpBin), &sh.full[buf]);
+    if (more) bulk_copy(&sh.ahead[buf], p.bins + b + p.nbuf, 16u, &sh.full[buf]);
 }
 
 __device__ __forceinline__ void cta_init(CtaShared &sh) {
@@ -790,7 +794,7 @@ __device__ __forceinline__ void begin_item(const TravParams &p, uint8_t *smem, C
     const int64_t row0 = tile * p.R;
     const int rows = (int)(p.n - row0 < (int64_t)p.R ? p.n - row0 : (int64_t)p.R);
     const int G = (rows + 31) >> 5;
-    if (tid == 0) {
+    if (tid < 32) {
         int b0 = 0, b1 = p.n_bins;
         if (p.n_splits > 1 && p.n_splits == p.n_passes) {
             const FpPass ps = p.passes[split];
@@ -800,14 +804,19 @@ __device__ __forceinline__ void begin_item(const TravParams &p, uint8_t *smem, C
             b0 = split * p.split_bins + min(split, p.split_more);
             b1 = b0 + p.split_bins + (split < p.split_more ? 1 : 0);
         }
-        sh.bin0 = b0;
-        sh.bin1 = b1;
-        sh.tile = tile;
-        uint32_t ph = 0;
-        for (int i = 0; i < FP_NBUF; ++i) ph |= ((uint32_t)sh.issued[i] & 1u) << i;
-        sh.phases = ph;
-        for (int i = 0; i < nbuf && b0 + i < b1; ++i)
-            stage_bin(p, sh, b0 + i, p.bins[b0 + i], i, smem + hbuf0 + i * p.head_smem);
+        if (tid == 0) {
+            sh.bin0 = b0;
+            sh.bin1 = b1;
+            sh.tile = tile;
+            uint32_t ph = 0;
+            for (int i = 0; i < FP_NBUF; ++i) ph |= ((uint32_t)sh.issued[i] & 1u) << i;
+            sh.phases = ph;
+        }
+        __syncwarp();
+        if (tid < nbuf && b0 + tid < b1) {  // a lane per buffer, so that the records' latencies overlap
+            const FpBin bn = p.bins[b0 + tid];
+            stage_bin(p, sh, b0 + tid, bn.head_off, bn.head_bytes, tid, smem + hbuf0 + tid * p.head_smem);
+        }
     }
     {
         // lane = row of a slab, 16 features at a time: loads along the row,
@@ -1067,8 +1076,8 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
         if (lane == 0) {
             const int done = atomicAdd(&sh.done[buf], 1);
             if (done == nwarps - 1 && b + nbuf < sh.bin1 && !*(volatile int *)&sh.abort) {
-                const FpBin next = p.bins[b + nbuf];
-                stage_bin(p, sh, b + nbuf, next, buf, smem + hbuf0 + buf * p.head_smem);
+                const uint4 next = sh.ahead[buf];
+                stage_bin(p, sh, b + nbuf, next.x, next.y, buf, smem + hbuf0 + buf * p.head_smem);
             }
         }
         __syncwarp();
