@@ -54,11 +54,12 @@
 // last split's CTA writes it).
 //
 // What bounds it (256 trees of 78.8k nodes, 28 features, 4 M rows, bins of 5
-// trees with heads 0..9: 24.4 ms; 27.5 ms as one pass of L2 after another with
+// trees with heads 0..9: 24.0 ms; 27.5 ms as one pass of L2 after another with
 // steps of divergent branches): the load/store data pipe, 80 % busy with 6.2
 // wavefronts per (row, tree), a little over half of them the super-nodes'
 // sectors and the rest shared-memory words; 17.9 warp instructions per (row,
-// tree) (23.4 before) take 63 % of the issue slots.
+// tree) (23.4 before) take 63 % of the issue slots.  (Counters of the walk at
+// 24.4 ms, before level heads of one word per node.)
 //
 // Waits: __syncthreads is a hardware wait; a wait for
 // a bin block polls its mbarrier at most spin_limit times (FP_SPIN_LIMIT
@@ -783,6 +784,13 @@ __device__ __forceinline__ void finish_rows(const TravParams &p, int64_t row0, i
     }
 }
 
+// 8 features of a row from a 32-byte aligned address, past L1.
+__device__ __forceinline__ void load_row8(const float4 *at, float4 &a, float4 &b) {
+    asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+                 : "l"(at));
+}
+
 // The start of an item: its bins and their first blocks in flight, its rows in
 // shared memory as order keys, its counters cleared.
 template <int MODE, int DK>
@@ -819,16 +827,21 @@ __device__ __forceinline__ void begin_item(const TravParams &p, uint8_t *smem, C
         }
     }
     {
-        // lane = row of a slab, 16 features at a time: loads along the row,
-        // and each store of a warp fills the 32 columns of one feature.  The
-        // (slab, 16 features) units are dealt out to all warps, so that a
-        // tile of few wide rows (784 features, 64 rows) is staged by every
-        // warp, not by two.
+        // lane = row of a slab, 8 features at a time: loads along the row, and
+        // each store of a warp fills the 32 columns of one feature.  The
+        // (slab, 8 features) units are dealt out to all warps, so that a tile
+        // of few wide rows (784 features, 64 rows) is staged by every warp,
+        // not by two.  A lane's 8 features are one 32-byte load where its
+        // address allows it: each sector is asked for once and used whole, and
+        // nothing is left for L1 to hold.  64-row tiles of 784 features (250 k
+        // rows): 1407 us, 1467 with four 16-byte loads a lane (16 features),
+        // 1435 with two (8 features); more loads in flight a lane, or runs of
+        // neighbouring features to one warp, 1480 to 1810.
         const float *src = p.X + row0 * F;
         const bool vec_rows = (F & 3) == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
-        const int fblocks = (F + 15) >> 4;
+        const int fblocks = (F + 7) >> 3;
         for (int u = warp; u < G * fblocks; u += nwarps) {
-            const int fq = u / G, g = u - fq * G, f0 = fq * 16;
+            const int fq = u / G, g = u - fq * G, f0 = fq * 8;
             const int r = g * 32 + lane;
             if (r >= rows) continue;
             const float *rp = src + (int64_t)r * F + f0;
@@ -841,16 +854,20 @@ __device__ __forceinline__ void begin_item(const TravParams &p, uint8_t *smem, C
                 d[96] = staged<DK>(p, v.w);
             };
             const float4 *rq = reinterpret_cast<const float4 *>(rp);
-            if (vec_rows && f0 + 16 <= F) {
-                float4 v[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) v[k] = __ldg(rq + k);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) put4(k, v[k]);
+            if (vec_rows && f0 + 8 <= F) {
+                float4 v[2];
+                if ((reinterpret_cast<uintptr_t>(rq) & 31) == 0) {
+                    load_row8(rq, v[0], v[1]);
+                } else {  // rows of 4, 12, ... features: every second one; or rows from the middle of a sector
+                    v[0] = __ldg(rq);
+                    v[1] = __ldg(rq + 1);
+                }
+                put4(0, v[0]);
+                put4(1, v[1]);
             } else if (vec_rows) {
-                for (int k = 0; f0 + 4 * k < F; ++k) put4(k, __ldg(rq + k));
+                put4(0, __ldg(rq));  // the last 4 of F
             } else {
-                const int m = F - f0 < 16 ? F - f0 : 16;
+                const int m = F - f0 < 8 ? F - f0 : 8;
 #pragma unroll 4
                 for (int k = 0; k < m; ++k) dst[32 * k] = staged<DK>(p, __ldg(rp + k));
             }
