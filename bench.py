@@ -609,7 +609,7 @@ def run_packed(args, ws, rank, local):
         "plain_baseline": plain,
         "packed_vs_plain": (value / ws / plain["value"]) if plain else None,
         "e2e": e2e,
-        "gpu_launches": args.steps,
+        "gpu_launches": args.steps,  # at least: a call of some waves and a tail is two launches
         # single launches timed one by one after the timed region: median and spread
         "launch_ms": {"median": statistics.median(per_launch_ms), "min": min(per_launch_ms),
                       "max": max(per_launch_ms), "n": len(per_launch_ms)},
