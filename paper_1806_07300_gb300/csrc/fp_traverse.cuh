@@ -277,6 +277,18 @@ struct LaneTask {
     int bad;
 };
 
+// A lane before its first task.  The deep step's reads of the row are not
+// predicated, so the row that such a lane reads (and makes nothing of) is
+// one of the tile's own: the first, at `base`.
+__host__ __device__ __forceinline__ LaneTask idle_task(uint32_t base) {
+    LaneTask L;
+    L.ref = FP_NO_TASK;
+    L.xb = base;
+    L.rt = 0;
+    L.bad = 0;
+    return L;
+}
+
 // A finished task's memory read whose result is not used at once: the leaf's
 // value on its way to the row's sum (values mode), or its leaf id on its way
 // to the output (parity mode).  Used one step later, when it has arrived; a
@@ -991,12 +1003,8 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
     begin_item<MODE, DK>(p, smem, sh, tile, split, hbuf0);
     __syncthreads();
 
-    LaneTask L;
-    L.ref = FP_NO_TASK;
-    L.xb = 0;
-    L.rt = 0;
-    L.bad = 0;
-    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    LaneTask L = idle_task(base);
+    uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // feature 0 in every slot
     Pending pend, hpend;  // of the last deep step, of the last burst
     pend.on = hpend.on = false;
     pend.at = hpend.at = 0;
