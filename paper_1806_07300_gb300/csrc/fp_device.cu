@@ -68,7 +68,11 @@ int cuda_fail(cudaError_t e, const char *what) {
 
 // Per-call scratch comes from the device's stream-ordered memory pool
 // (cudaMallocAsync), which CUDA-graph capture turns into graph memory nodes.
-// The first use on a device keeps freed blocks in the pool between calls.
+// The first use on a device keeps freed blocks in the pool between calls.  A
+// failed allocation is reported by the return code alone: the runtime's own
+// record of it (the thread's last error) is cleared, since the caller may go
+// on without scratch.  An injected failure asks the runtime for more than any
+// device has, so that it leaves the state that a real one does.
 int scratch_alloc(int device, void **out, size_t bytes, cudaStream_t s) {
     {
         std::lock_guard<std::mutex> lk(g_pool_mu);
@@ -83,9 +87,13 @@ int scratch_alloc(int device, void **out, size_t bytes, cudaStream_t s) {
             g_pool_ready[device] = 1;
         }
     }
-    if (injected_alloc_failure("cudaMallocAsync(scratch)")) return FP_ENOMEM;
-    cudaError_t e = cudaMallocAsync(out, bytes, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(scratch)");
+    const bool injected = injected_alloc_failure("cudaMallocAsync(scratch)");
+    cudaError_t e = cudaMallocAsync(out, injected ? (size_t)1 << 60 : bytes, s);
+    if (injected && e == cudaSuccess) cudaFreeAsync(*out, s);  // not on any device there is
+    if (injected || e != cudaSuccess) {
+        cudaGetLastError();
+        return injected ? FP_ENOMEM : cuda_fail(e, "cudaMallocAsync(scratch)");
+    }
     return FP_OK;
 }
 
@@ -454,12 +462,19 @@ void set_shape(TravParams &p, const Shape &sh) {
     p.split_more = p.n_bins % sh.S;
 }
 
+// A kernel launch that returns its own result: the thread's last error, which
+// is all that <<<>>> leaves, may be that of an earlier call.
+template <class Params>
+cudaError_t launch(void (*kern)(Params), int64_t ctas, int threads, size_t smem, cudaStream_t s, const Params &p) {
+    void *args[] = {const_cast<Params *>(&p)};
+    return cudaLaunchKernel(reinterpret_cast<const void *>(kern), dim3((unsigned)ctas), dim3((unsigned)threads), args,
+                            smem, s);
+}
+
 // Launch one part of a call, shaped by set_shape.
 template <int MODE>
 cudaError_t launch_part(const fp_device_forest *f, const TravParams &p, int32_t grid, size_t smem, cudaStream_t s) {
-    const int64_t ctas = std::min<int64_t>(p.n_items, grid);
-    traverse_kernel<MODE>(f)<<<(unsigned)ctas, f->threads, smem, s>>>(p);
-    return cudaGetLastError();
+    return launch(traverse_kernel<MODE>(f), std::min<int64_t>(p.n_items, grid), f->threads, smem, s, p);
 }
 
 // Whether a call on this stream may take scratch that it would not need
@@ -467,7 +482,9 @@ cudaError_t launch_part(const fp_device_forest *f, const TravParams &p, int32_t 
 // limits what can be done with the graph.
 bool may_split(cudaStream_t s) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st == cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the call goes on: without scratch
+    return false;
 }
 
 // Scratch of a part whose splits add up in global memory: acc_per_row bytes of
@@ -1032,8 +1049,7 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * warps, smem);
     if (e == cudaSuccess) {
         const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(bp.item_begin[m], (int64_t)per_sm * sms));
-        kern<<<(unsigned)grid, 32 * warps, smem, s>>>(bp);
-        e = cudaGetLastError();
+        e = launch(kern, grid, 32 * warps, smem, s, bp);
     }
     cudaFreeAsync(scratch, s);
     if (e != cudaSuccess) return cuda_fail(e, "fp_predict_batched");
