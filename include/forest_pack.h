@@ -226,10 +226,11 @@ int fp_configure(fp_device_forest *forest, const fp_pack_params *params);
  *              or NULL
  * Asynchronous on `stream`; X must stay valid and the outputs untouched until
  * the stream reaches this work.  Calls on different streams may overlap.  A
- * small batch may use stream-ordered scratch (a forest of one pass does
- * without when there is none, or when the stream is being captured).
- * Errors: FP_EINVAL, FP_ENOMEM (scratch of a forest of several passes),
- * FP_ECUDA. */
+ * small batch may use stream-ordered scratch for the classes (a forest of one
+ * pass does without when there is none, or when the stream is being captured;
+ * votes alone, out_class NULL, never need any).
+ * Errors: FP_EINVAL, FP_ENOMEM (scratch for the classes of a forest of several
+ * passes), FP_ECUDA. */
 int fp_predict(const fp_device_forest *forest, const float *X, int64_t n, uint32_t *out_votes, int32_t *out_class,
                void *stream);
 
@@ -251,7 +252,8 @@ int fp_predict(const fp_device_forest *forest, const float *X, int64_t n, uint32
  * stream capture.  All calls on a device share its one array, which keeps
  * the last call's contents; each call clears the part it uses.  Calls whose
  * work overlaps on the GPU (for instance on two streams) race on the array
- * and must be ordered by the caller.  Nothing is allocated or freed: no
+ * and must be ordered by the caller, unless they ask for votes alone
+ * (out_class NULL), which do not touch it.  Nothing is allocated or freed: no
  * cudaMalloc, cudaFree, cudaMallocAsync or library allocator. */
 int fp_predict_noalloc(const fp_device_forest *forest, const float *X, int64_t n, uint32_t *out_votes,
                        int32_t *out_class, void *stream);

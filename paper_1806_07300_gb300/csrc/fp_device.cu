@@ -638,7 +638,11 @@ namespace {
 
 // fp_predict and fp_predict_noalloc: scratch_for(bytes, &ptr) supplies the
 // scratch of a part, release(ptr) takes it back.  A part that gets none runs
-// unsplit where the forest has one pass, or where `whole` says so.
+// unsplit where the forest has one pass, or where `whole` says so.  Votes
+// without classes take no scratch: the splits add up in the caller's votes and
+// nothing is left to do after the last of them.  So such calls cannot fail for
+// memory, put no memory node into a captured graph, and overlap freely when
+// they are fp_predict_noalloc's.
 template <class Scratch, class Release>
 int predict_votes(const fp_device_forest *f, const float *X, int64_t n, uint32_t *out_votes, int32_t *out_class,
                   cudaStream_t s, bool split, bool whole, Scratch scratch_for, Release release) {
@@ -651,9 +655,10 @@ int predict_votes(const fp_device_forest *f, const float *X, int64_t n, uint32_t
         // the splits add up in scratch, or, where that would be large, in the
         // caller's votes (a second memset)
         const int64_t vote_bytes = 4 * (int64_t)h.n_classes;
-        const bool in_votes = votes && pt.n * vote_bytes > (4 << 20);
-        size_t acc_bytes;
-        const size_t bytes = scratch_bytes(pt, in_votes ? 0 : vote_bytes, &acc_bytes);
+        const bool votes_alone = !out_class;
+        const bool in_votes = votes_alone || (votes && pt.n * vote_bytes > (4 << 20));
+        size_t acc_bytes = 0;
+        const size_t bytes = votes_alone ? 0 : scratch_bytes(pt, in_votes ? 0 : vote_bytes, &acc_bytes);
         void *scratch = nullptr;
         if (bytes) {
             const int rc = scratch_for(bytes, &scratch);
@@ -668,8 +673,8 @@ int predict_votes(const fp_device_forest *f, const float *X, int64_t n, uint32_t
         if (p.n_splits > 1) {
             uint8_t *sc = static_cast<uint8_t *>(scratch);
             p.acc = in_votes ? votes : reinterpret_cast<uint32_t *>(sc);
-            p.tile_done = reinterpret_cast<uint32_t *>(sc + acc_bytes);
-            e = cudaMemsetAsync(scratch, 0, bytes, s);
+            p.tile_done = votes_alone ? nullptr : reinterpret_cast<uint32_t *>(sc + acc_bytes);
+            if (bytes) e = cudaMemsetAsync(scratch, 0, bytes, s);
             if (e == cudaSuccess && in_votes) e = cudaMemsetAsync(votes, 0, (size_t)(pt.n * vote_bytes), s);
         }
         if (e == cudaSuccess) e = launch_part<FP_MODE_VOTES>(f, p, f->grid_votes, f->smem_votes, s);
@@ -696,7 +701,7 @@ extern "C" int fp_predict(const fp_device_forest *f, const float *X, int64_t n, 
     if (rc) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     return predict_votes(
-        f, X, n, out_votes, out_class, s, may_split(s), false,
+        f, X, n, out_votes, out_class, s, !out_class || may_split(s), false,
         [&](size_t bytes, void **out) { return scratch_alloc(f->device, out, bytes, s); },
         [&](void *ptr) { cudaFreeAsync(ptr, s); });
 }

@@ -46,7 +46,8 @@
 //   5. writes votes and the argmax class (lowest class on ties).  With one
 //      split the tile's votes are complete in shared memory; with several, they
 //      are added to a global accumulator and the CTA that finishes a tile's
-//      last split takes the argmax (per-tile counter, no waiting).
+//      last split takes the argmax (per-tile counter, no waiting; no counter
+//      and no argmax when votes alone are asked for).
 // Parity mode writes the leaf id reached in every (observation, tree)
 // instead of voting.  Values mode (forests with real leaf values: regression
 // and boosted trees) adds the leaf's value to a float per row instead, and
@@ -105,7 +106,7 @@ struct TravParams {
     int32_t *out_class;       // may be NULL
     int32_t *out_leaf;        // parity mode
     uint32_t *acc;            // several splits: vote accumulator
-    uint32_t *tile_done;      // several splits: per-tile counter of finished ones
+    uint32_t *tile_done;      // several splits: per-tile counter of finished ones (NULL: votes alone are asked for)
     int32_t *status;          // device status word
     const float *leaf_val;    // forests with leaf values: value of each leaf slot
     uint32_t n_vals;          // slots in leaf_val
@@ -796,6 +797,22 @@ __device__ __forceinline__ void finish_rows(const TravParams &p, int64_t row0, i
     }
 }
 
+// A split's votes for class 0, where votes alone are asked for: no CTA looks at
+// the tile again, so each split adds its own (its trees less the votes for the
+// others).  Not inlined, to keep the walks of the kernels that call it as they
+// are.
+__device__ __noinline__ void add_class0(const TravParams &p, const CtaShared &sh, uint32_t at0, int64_t row0,
+                                        int rows) {
+    const int end = sh.bin1 < p.n_bins ? p.bins[sh.bin1].first_tree : p.T;
+    const uint32_t trees = (uint32_t)(end - p.bins[sh.bin0].first_tree);
+    for (int rr = threadIdx.x; rr < rows; rr += blockDim.x) {
+        const uint32_t at = at0 + (uint32_t)(rr >> 5) * p.slab + ((uint32_t)p.F << 7) + (uint32_t)(rr & 31) * 4u;
+        uint32_t rest = trees;
+        for (int c = 1; c < p.C; ++c) rest -= lds(at + ((uint32_t)c << 7));
+        if (rest) atomicAdd(p.acc + (row0 + rr) * p.C, rest);
+    }
+}
+
 // 8 features of a row from a 32-byte aligned address, past L1.
 __device__ __forceinline__ void load_row8(const float4 *at, float4 &a, float4 &b) {
     asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
@@ -956,7 +973,11 @@ __device__ __forceinline__ void end_item(const TravParams &p, uint8_t *smem, Cta
                 const uint32_t v = rr < nrows ? lds(counter(rr, c)) : 0u;
                 if (v) atomicAdd(p.acc + (base + rr) * C + c, v);
             }
-            if (last_split()) finish_rows(p, base, nrows);
+            if (p.tile_done) {
+                if (last_split()) finish_rows(p, base, nrows);
+            } else {
+                add_class0(p, sh, at0, base, nrows);
+            }
         }
     }
 }

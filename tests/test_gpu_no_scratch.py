@@ -1,6 +1,8 @@
 """Calls that would split a small batch's bins over the GPU, and then find no
 scratch to add the splits up in.  The failure is injected as a request that
 the runtime itself refuses, so the thread is left as a real failure leaves it."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -61,4 +63,100 @@ def test_values_without_scratch(n):
     assert df.sync_status() == fp.FP_OK
     err = np.abs(out.cpu().numpy().astype(np.float64) - ref["out"])
     assert np.all(err <= oracle.value_tolerance(F, ref["abs"]))
+    df.release()
+
+
+def _multi_pass(tiny_forest):
+    pf = fp.fp_pack_forest(tiny_forest, bin_size=2, interleave_depth=2, pass_bytes=2048)
+    assert pf.info()["passes"] > 1
+    return fp.fp_upload(pf)
+
+
+def _node_types(graph):
+    """Types of the nodes of a captured graph that was kept (CUgraphNodeType)."""
+    drv, g = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(graph.raw_cuda_graph())
+    n = ctypes.c_size_t(0)
+    assert drv.cuGraphGetNodes(g, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert drv.cuGraphGetNodes(g, nodes, ctypes.byref(n)) == 0
+    types = []
+    for node in nodes:
+        t = ctypes.c_int(-1)
+        assert drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(t)) == 0
+        types.append(t.value)
+    return types
+
+
+MEMORY_NODES = {10, 11}  # CU_GRAPH_NODE_TYPE_MEM_ALLOC, CU_GRAPH_NODE_TYPE_MEM_FREE
+
+
+@pytest.mark.parametrize("n", [1, 33, 3000])
+def test_votes_alone_need_no_scratch(tiny_forest, tiny_rows, n):
+    """A forest of several passes, votes without classes: no allocation is
+    made (an injected failure waits for the next one)."""
+    X = np.ascontiguousarray(tiny_rows[0][:n])
+    df = _multi_pass(tiny_forest)
+    Xd = torch.from_numpy(X).cuda()
+    want = oracle.predict(tiny_forest, X)["votes"]
+    fp.fp_inject_fault(None, fp.FP_FAULT_ALLOC, 1)
+    v, _ = df.predict(Xd, classes=False)
+    with pytest.raises(fp.FPError):
+        fp.fp_upload(fp.fp_pack_forest(tiny_forest))
+    w = torch.full((n, tiny_forest.n_classes), -1, dtype=torch.int32, device="cuda")
+    fp.fp_predict_noalloc(df, Xd, w, None)
+    assert df.sync_status() == fp.FP_OK
+    np.testing.assert_array_equal(v.cpu().numpy().astype(np.uint32), want)
+    np.testing.assert_array_equal(w.cpu().numpy().astype(np.uint32), want)
+    df.release()
+
+
+@pytest.mark.parametrize("several_passes", [False, True])
+@pytest.mark.parametrize("classes", [False, True])
+def test_memory_nodes_under_capture(tiny_forest, tiny_rows, several_passes, classes):
+    """Under capture a small batch makes memory nodes only for the classes of
+    a forest of several passes."""
+    X = np.ascontiguousarray(tiny_rows[0][:64])
+    df = _multi_pass(tiny_forest) if several_passes else fp.fp_upload(
+        fp.fp_pack_forest(tiny_forest, bin_size=1, interleave_depth=3, pass_bytes=-1))
+    Xd = torch.from_numpy(X).cuda()
+    v = torch.empty((64, tiny_forest.n_classes), dtype=torch.int32, device="cuda")
+    c = torch.empty((64,), dtype=torch.int32, device="cuda") if classes else None
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    fp.fp_predict(df, Xd, v, c, stream=s)
+    s.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=s):
+        fp.fp_predict(df, Xd, v, c, stream=torch.cuda.current_stream())
+    assert bool(MEMORY_NODES & set(_node_types(g))) == (several_passes and classes)
+    g.instantiate()
+    v.fill_(-1)
+    g.replay()
+    torch.cuda.synchronize()
+    ref = oracle.predict(tiny_forest, X)
+    np.testing.assert_array_equal(v.cpu().numpy().astype(np.uint32), ref["votes"])
+    if classes:
+        np.testing.assert_array_equal(c.cpu().numpy(), ref["cls"])
+    df.release()
+
+
+def test_noalloc_votes_alone_overlap(tiny_forest, tiny_rows):
+    """fp_predict_noalloc for votes alone leaves the shared array alone, so
+    calls on two streams do not meet in it."""
+    df = _multi_pass(tiny_forest)
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    Xs = [np.ascontiguousarray(tiny_rows[0][k * 500:k * 500 + 500]) for k in range(2)]
+    Xd = [torch.from_numpy(x).cuda() for x in Xs]
+    vs = [[torch.full((500, tiny_forest.n_classes), -1, dtype=torch.int32, device="cuda") for _ in range(20)]
+          for _ in range(2)]
+    torch.cuda.synchronize()
+    for i in range(20):
+        for k, s in enumerate(streams):
+            fp.fp_predict_noalloc(df, Xd[k], vs[k][i], None, stream=s)
+    torch.cuda.synchronize()
+    assert df.sync_status() == fp.FP_OK
+    for k in range(2):
+        want = oracle.predict(tiny_forest, Xs[k])["votes"]
+        for v in vs[k]:
+            np.testing.assert_array_equal(v.cpu().numpy().astype(np.uint32), want)
     df.release()
