@@ -811,6 +811,9 @@ extern "C" int fp_predict_noalloc(const fp_device_forest *f, const float *X, int
                          (long long)n, bytes, FP_NOALLOC_SCRATCH_BYTES);
             return FP_EINVAL;
         }
+        void *scratch;  // the address is looked up whether this call needs the array or not
+        rc = noalloc_scratch(f->device, &scratch);
+        if (rc) return rc;
     }
     return predict_votes(
         f, X, n, out_votes, out_class, s, false, true,

@@ -2,6 +2,9 @@
 scratch to add the splits up in.  The failure is injected as a request that
 the runtime itself refuses, so the thread is left as a real failure leaves it."""
 import ctypes
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -12,6 +15,7 @@ import paper_1806_07300_gb300 as fp
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -160,3 +164,28 @@ def test_noalloc_votes_alone_overlap(tiny_forest, tiny_rows):
         for v in vs[k]:
             np.testing.assert_array_equal(v.cpu().numpy().astype(np.uint32), want)
     df.release()
+
+
+def test_noalloc_small_call_captured_after_a_large_one(tiny_forest, tiny_rows):
+    """The first call on a device looks up the array, also when it is large
+    enough to need none; a small classes-only call can then be captured.  A
+    process of its own, since the address is kept."""
+    code = """
+import numpy as np, torch, datagen, oracle
+import paper_1806_07300_gb300 as fp
+F, X = datagen.forest("tiny"), datagen.test_rows("tiny")[0]
+df = fp.fp_upload(fp.fp_pack_forest(F, bin_size=2, interleave_depth=2, pass_bytes=2048))
+Xd = torch.from_numpy(np.tile(X, (16, 1))).cuda()
+n = Xd.shape[0]
+v, c = (torch.empty(s, dtype=torch.int32, device="cuda") for s in ((n, F.n_classes), (n,)))
+fp.fp_predict_noalloc(df, Xd, v, c)
+torch.cuda.synchronize()
+s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+with torch.cuda.graph(g, stream=s):
+    fp.fp_predict_noalloc(df, Xd[:64], None, c[:64], stream=torch.cuda.current_stream())
+c.fill_(-1)
+g.replay()
+torch.cuda.synchronize()
+assert np.array_equal(c[:64].cpu().numpy(), oracle.predict(F, X[:64])["cls"])
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT, timeout=600)
