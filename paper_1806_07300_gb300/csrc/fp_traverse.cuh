@@ -1113,7 +1113,11 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
                           LEAVES ? (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11) : xb);
                 tail += __popc(pm);
                 __syncwarp();
-                deep_finish<MODE, DK>(p, L, pend, w);
+                // where nearly all paths end in the heads, most bursts find no
+                // lane with a task: 16 trees of 80 nodes, 400,000 rows: 87.0 us
+                // with the step taken all the same, 80.0 without; the vote
+                // costs forests of deep trees 0.3 %
+                if (__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) deep_finish<MODE, DK>(p, L, pend, w);
                 pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
             }
         }
