@@ -292,8 +292,12 @@ __host__ __device__ __forceinline__ LaneTask idle_task(uint32_t base) {
 
 // A finished task's memory read whose result is not used at once: the leaf's
 // value on its way to the row's sum (values mode), or its leaf id on its way
-// to the output (parity mode).  Used one step later, when it has arrived; a
-// use at once stalls the warp for a whole L2 latency in nearly every step.
+// to the output (parity mode).  Used right before the next deep step, which
+// waits for its super-nodes there anyway; a use at once stalls the warp for a
+// whole L2 latency in nearly every step, and one before the head walk between
+// two steps waits where the walk could have hidden it (leaf ids of 64 trees,
+// 100-feature rows, 100,000 rows: 160 -> 146 us, 155 before leaf ids were used
+// late at all; 128 regression trees, 1 M rows: 2856 -> 2769 us).
 struct Pending {
     bool on;
     uint32_t at;      // values: xb; parity: rt
@@ -314,18 +318,19 @@ __device__ __forceinline__ void add_value(const TravParams &p, uint32_t xb, floa
     add_shared(xb + ((uint32_t)p.F << 7), v);
 }
 
-__device__ __forceinline__ void put_leaf(const TravParams &p, const CtaShared &sh, uint32_t rt, int32_t leaf_id) {
-    p.out_leaf[(sh.tile * p.R + (rt & 2047u)) * p.T + (rt >> 11)] = leaf_id;
+// Parity mode; leaves: the output from the tile's first row on.
+__device__ __forceinline__ void put_leaf(const TravParams &p, int32_t *leaves, uint32_t rt, int32_t leaf_id) {
+    leaves[(uint64_t)(rt & 2047u) * (uint32_t)p.T + (rt >> 11)] = leaf_id;
 }
 
 template <int MODE>
-__device__ __forceinline__ void settle(const TravParams &p, const CtaShared &sh, Pending &pend) {
+__device__ __forceinline__ void settle(const TravParams &p, int32_t *leaves, Pending &pend) {
     if (MODE == FP_MODE_VOTES) return;
     if (pend.on) {
         if (MODE == FP_MODE_VALUES)
             add_value(p, pend.at, __uint_as_float(pend.word));
         else
-            put_leaf(p, sh, pend.at, (int32_t)pend.word);
+            put_leaf(p, leaves, pend.at, (int32_t)pend.word);
     }
     pend.on = false;
 }
@@ -656,7 +661,7 @@ __device__ __forceinline__ void head_walks(const TravParams &p, uint32_t blk, ui
 template <int MODE, bool KEYS, int HK>
 __device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, CtaShared &sh, const FpBin &bn,
                                            uint32_t blk, uint32_t exits, int buf, int rows, int G, uint32_t inv_g,
-                                           int &bad) {
+                                           int32_t *leaves, int &bad) {
     const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     // runs of 32 trees, shorter when the bin would leave warps without one
     const int run = max(1, min(32, bn.width * G / nwarps));
@@ -678,7 +683,7 @@ __device__ __forceinline__ void walk_heads(const TravParams &p, uint32_t base, C
                 sum += __uint_as_float(lds(at));  // the exits hold the leaves' values themselves
             } else if (MODE == FP_MODE_LEAVES) {
                 if (my)
-                    put_leaf(p, sh, (uint32_t)r | ((uint32_t)(bn.first_tree + k) << 11),
+                    put_leaf(p, leaves, (uint32_t)r | ((uint32_t)(bn.first_tree + k) << 11),
                              p.pheads[(bn.phead_off >> 2) + ((at - exits) >> 2)]);
             } else {
                 const uint32_t cls = lds(at) & 0x7FFFFFFFu;
@@ -1020,13 +1025,14 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
     const int64_t row0 = tile * R;
     const int rows = (int)(p.n - row0 < (int64_t)R ? p.n - row0 : (int64_t)R);
     const int G = (rows + 31) >> 5;  // slabs in use
+    int32_t *const leaves = LEAVES ? p.out_leaf + row0 * p.T : nullptr;
 
     begin_item<MODE, DK>(p, smem, sh, tile, split, hbuf0);
     __syncthreads();
 
     LaneTask L = idle_task(base);
     uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // feature 0 in every slot
-    Pending pend, hpend;  // of the last deep step, of the last burst
+    Pending pend, hpend;  // of the last deep step, of the last burst (values mode)
     pend.on = hpend.on = false;
     pend.at = hpend.at = 0;
     pend.word = hpend.word = 0;
@@ -1063,20 +1069,19 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
         const uint32_t blk = base + hbuf0 + (uint32_t)(buf * p.head_smem);
         const uint32_t exits = blk + (uint32_t)(nranks * stride * (levels == 2 ? 16 : (levels == 3 ? 4 : 8)));
 
-        if (HEADS) walk_heads<MODE, D3, HK>(p, base, sh, bn, blk, exits, buf, rows, G, inv_g, L.bad);
+        if (HEADS) walk_heads<MODE, D3, HK>(p, base, sh, bn, blk, exits, buf, rows, G, inv_g, leaves, L.bad);
         const int units = bn.width * G;
         if (!HEADS) {
             for (;;) {
                 // deep steps until the ring runs low
                 if (!carried) ld_super(p.deep, L.ref, w);
                 carried = false;
-                settle<MODE>(p, sh, pend);
-                settle<MODE>(p, sh, hpend);
+                settle<MODE>(p, leaves, hpend);
                 while (__any_sync(0xffffffffu, tail - head > p.refill)) {
+                    settle<MODE>(p, leaves, pend);
                     deep_finish<MODE, DK>(p, L, pend, w);
                     pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
                     ld_super(p.deep, L.ref, w);
-                    settle<MODE>(p, sh, pend);
                 }
                 int unit = 0;
                 if (lane == 0) unit = atomicAdd(&sh.next[buf], 1);
@@ -1095,9 +1100,9 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
                     const uint32_t cls = er & 0x7FFFFFFFu;
                     if (LEAVES) {
                         L.bad |= !ok;
-                        hpend.on = ok;
-                        hpend.at = (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11);
-                        if (ok) hpend.word = (uint32_t)__ldg(p.pheads + (bn.phead_off >> 2) + ((at - exits) >> 2));
+                        if (ok)
+                            put_leaf(p, leaves, (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11),
+                                     __ldg(p.pheads + (bn.phead_off >> 2) + ((at - exits) >> 2)));
                     } else if (VALUES) {
                         L.bad |= cls >= p.n_vals;
                         hpend.on = cls < p.n_vals;
@@ -1113,6 +1118,7 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
                           LEAVES ? (uint32_t)r2 | ((uint32_t)(bn.first_tree + uk) << 11) : xb);
                 tail += __popc(pm);
                 __syncwarp();
+                settle<MODE>(p, leaves, pend);
                 // where nearly all paths end in the heads, most bursts find no
                 // lane with a task: 16 trees of 80 nodes, 400,000 rows: 87.0 us
                 // with the step taken all the same, 80.0 without; the vote
@@ -1136,6 +1142,7 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
         // bin would cost most warps an L2 latency for nothing
         carried = units < nwarps;
         if (!HEADS && !carried && __any_sync(0xffffffffu, L.ref != FP_NO_TASK)) {
+            settle<MODE>(p, leaves, pend);
             deep_finish<MODE, DK>(p, L, pend, w);
             pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
         }
@@ -1148,11 +1155,11 @@ __device__ __forceinline__ void run_item(const TravParams &p, int64_t tile, int 
         pop_tasks<MODE>(p, base, ring, head, tail, L, lt_mask);
         if (!__any_sync(0xffffffffu, L.ref != FP_NO_TASK)) break;
         ld_super(p.deep, L.ref, w);
-        settle<MODE>(p, sh, pend);
+        settle<MODE>(p, leaves, pend);
         deep_finish<MODE, DK>(p, L, pend, w);
     }
-    settle<MODE>(p, sh, pend);
-    settle<MODE>(p, sh, hpend);
+    settle<MODE>(p, leaves, pend);
+    settle<MODE>(p, leaves, hpend);
     if (L.bad) report(p.status, FP_ERR_FLAG_DEVICE);
     __syncthreads();
 
