@@ -206,7 +206,8 @@ const void *fp_packed_image(const fp_packed_forest *pf, int64_t *bytes);
 /* Copy a packed image to the current device on `stream` and return a
  * resident forest (library-owned until fp_release).  The call waits for the
  * copy to finish on `stream`, so the host image may be released once it
- * returns.  Errors: FP_EINVAL, FP_ENOMEM, FP_ECUDA, FP_EUNSUPPORTED (the
+ * returns.  A second form of the trees' heads, faster to walk, is made on the
+ * device where there is memory for it (about the heads' size).  Errors: FP_EINVAL, FP_ENOMEM, FP_ECUDA, FP_EUNSUPPORTED (the
  * launch does not fit shared memory). */
 int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_forest **out);
 
@@ -396,6 +397,8 @@ int fp_sync_status(const fp_device_forest *forest, void *stream);
  *                            device allocations made by fp_upload and by the
  *                            scratch of fp_predict / fp_predict_batched fail
  *                            with FP_ENOMEM (0 clears)
+ *   FP_FAULT_ALLOC_AFTER     forest ignored; those begin after `value`
+ *                            allocations that are left alone
  *   FP_FAULT_WAIT_LIMIT      a bin-block wait of this forest's kernels polls its
  *                            barrier at most `value` times (1 .. 2^24; the
  *                            default is 2^24) before recording FP_ETIMEOUT
@@ -409,6 +412,7 @@ int fp_sync_status(const fp_device_forest *forest, void *stream);
 #define FP_FAULT_ALLOC 1
 #define FP_FAULT_WAIT_LIMIT 2
 #define FP_FAULT_STALL_BIN_COPY 3
+#define FP_FAULT_ALLOC_AFTER 4
 int fp_inject_fault(fp_device_forest *forest, int32_t kind, int64_t value);
 
 /* Sizes of a resident forest (same fields as fp_packed_info_get). */

@@ -384,12 +384,13 @@ def fp_sync_status(forest: "DeviceForest", stream=None) -> int:
     return lib().fp_sync_status(forest.handle, _stream_ptr(stream))
 
 
-FP_FAULT_ALLOC, FP_FAULT_WAIT_LIMIT, FP_FAULT_STALL_BIN_COPY = 1, 2, 3
+FP_FAULT_ALLOC, FP_FAULT_WAIT_LIMIT, FP_FAULT_STALL_BIN_COPY, FP_FAULT_ALLOC_AFTER = 1, 2, 3, 4
 
 
 def fp_inject_fault(forest, kind: int, value: int) -> None:
     """Fault injection for failure-detection tests: FP_FAULT_ALLOC (forest may
-    be None) makes the next `value` device allocations fail with FP_ENOMEM;
+    be None) makes the next `value` device allocations fail with FP_ENOMEM,
+    or those after the next FP_FAULT_ALLOC_AFTER ones;
     FP_FAULT_WAIT_LIMIT bounds a bin-block wait to `value` polls;
     FP_FAULT_STALL_BIN_COPY=1 makes the forest's bin waits run out, so its
     launches record FP_ETIMEOUT (0 restores)."""

@@ -49,10 +49,15 @@ namespace {
 
 std::mutex g_pool_mu;
 std::vector<int> g_pool_ready;
-std::atomic<int64_t> g_fail_allocs{0};  // fault injection: device allocations still to fail
+std::atomic<int64_t> g_fail_allocs{0};  // fault injection: device allocations still to fail ...
+std::atomic<int64_t> g_pass_allocs{0};  // ... after this many that go through
 
 // true when fault injection takes this allocation
 bool injected_alloc_failure(const char *what) {
+    int64_t pass = g_pass_allocs.load();
+    while (pass > 0 && !g_pass_allocs.compare_exchange_weak(pass, pass - 1)) {
+    }
+    if (pass > 0) return false;
     int64_t k = g_fail_allocs.load();
     while (k > 0 && !g_fail_allocs.compare_exchange_weak(k, k - 1)) {
     }
@@ -125,8 +130,10 @@ void (*traverse_kernel_deep(const fp_device_forest *f))(TravParams) {
             default: return fp_traverse_kernel<MODE, 1, DK, 0, true>;
         }
     }
-    switch (f->levels) {  // unpaired level slots have float thresholds only, those of one word have keys only
-        case 1: return traverse_kernel_sized<MODE, DK, DK == 2 ? 1 : 0>(f);
+    switch (f->levels) {  // level slots of one word have keys only
+        case 1:
+            // with keys, only where the one-word heads found no memory: one build for every CTA size
+            return DK == 2 ? traverse_kernel_sized<MODE, 2, 1>(f) : fp_traverse_kernel<MODE, 1, DK == 2 ? 3 : DK, 1, false>;
         case 2: return traverse_kernel_sized<MODE, DK, 2>(f);
         case 3: return traverse_kernel_sized<MODE, DK, DK == 2 ? 0 : 3>(f);
         default: return traverse_kernel_sized<MODE, DK, 0>(f);
@@ -510,14 +517,14 @@ int check_device(const fp_device_forest *f) {
 }  // namespace
 
 // The one-word level heads of an uploaded forest (fp_compact_heads_kernel) and
-// their bins; the forest then walks those.  Waits for the stream.
+// their bins; the forest then walks those.  Waits for the stream.  FP_ENOMEM
+// leaves the forest with its packed heads, which serve every launch.
 static int compact_heads(fp_device_forest *f, cudaStream_t s) {
     const FpImageHeader &h = f->hdr;
     std::vector<FpBin> bins;
     try {
         bins = f->bins;
     } catch (const std::bad_alloc &) {
-        fp_set_error("fp_upload: out of host memory");
         return FP_ENOMEM;
     }
     const int32_t nodes = (1 << (h.depth + 1)) - 1;
@@ -531,8 +538,14 @@ static int compact_heads(fp_device_forest *f, cudaStream_t s) {
         largest = std::max<int32_t>(largest, (int32_t)b.head_bytes);
     }
     f->compact_bins_bytes = ((int64_t)(bins.size() * sizeof(FpBin)) + 255) & ~(int64_t)255;
-    cudaError_t e = cudaMalloc(&f->d_compact, (size_t)(f->compact_bins_bytes + off));
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(heads)");
+    cudaError_t e = cudaErrorMemoryAllocation;
+    if (!injected_alloc_failure("cudaMalloc(heads)"))
+        e = cudaMalloc(&f->d_compact, (size_t)(f->compact_bins_bytes + off));
+    if (e != cudaSuccess) {
+        f->d_compact = nullptr;
+        cudaGetLastError();
+        return cuda_fail(e, "cudaMalloc(heads)");
+    }
     e = cudaMemcpyAsync(f->d_compact, bins.data(), bins.size() * sizeof(FpBin), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(heads)");
     fp_compact_heads_kernel<<<(unsigned)bins.size(), 256, 0, s>>>(
@@ -600,7 +613,7 @@ extern "C" int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_for
     fit_costs(f);
     if (h->n_super > 0 && deep_kind(*h) >= 3 && f->levels != 0) {
         rc = compact_heads(f, s);
-        if (rc) goto fail;
+        if (rc && rc != FP_ENOMEM) goto fail;
     }
     rc = launch_setup(f, h->obs_tile, h->warps_per_cta, h->refill_lanes, h->bin_buffers);
     if (rc) goto fail;
@@ -877,6 +890,11 @@ extern "C" int fp_inject_fault(fp_device_forest *f, int32_t kind, int64_t value)
     case FP_FAULT_ALLOC:
         if (value < 0) break;
         g_fail_allocs.store(value);
+        if (value == 0) g_pass_allocs.store(0);
+        return FP_OK;
+    case FP_FAULT_ALLOC_AFTER:
+        if (value < 0) break;
+        g_pass_allocs.store(value);
         return FP_OK;
     case FP_FAULT_WAIT_LIMIT:
         if (!f || value < 1 || value > FP_SPIN_LIMIT) break;
