@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -937,29 +938,78 @@ extern "C" void fp_release(fp_device_forest *f) {
     delete f;
 }
 
-// The shape of one batch when no item of it is to take longer than `most`
-// nanoseconds: the splits, of a few numbers of them, whose items (as large as
-// `most` lets them be) take the least time together.
-static Shape shape_within(const fp_device_forest *f, int64_t n, int32_t max_R, double most) {
-    const int64_t nb = f->hdr.n_bins, top = std::min<int64_t>(max_R, (n + 31) / 32 * 32);
-    Shape best;
-    for (int64_t S = 1;; S = std::min(nb, S + 1 + S / 2)) {
-        const int64_t bins = (nb + S - 1) / S;
-        const double fixed = item_cost(f, 0, bins), per_row = item_cost(f, 1, bins) - fixed;
-        const double fit = std::max(32.0, std::min((most - fixed) / per_row, (double)top));
-        const int64_t R = (int64_t)fit / 32 * 32, tiles = (n + R - 1) / R;
-        const double item = item_cost(f, R, bins) + (S > 1 ? 1000.0 : 0.0);
-        // an item that is too long all the same counts for more
-        const double cost = (double)(tiles * S) * item * (item > most ? item / most : 1.0);
-        if (cost < best.cost) {
-            best.R = (int32_t)R;
-            best.S = (int32_t)S;
-            best.cost = cost;
+// One batch of a launch of several: the numbers of splits that it may be cut
+// into, with what the estimates need of each.  Formed once per call, since the
+// search below asks for a shape for every length of item: with the estimates
+// formed anew each time, 32 batches of a few rows kept the host planning for
+// as long as the launch itself takes.
+struct BatchCuts {
+    struct Cut {
+        int64_t S;
+        double fixed, per_row, inv_row, more;  // an item's time without rows, per row, and for adding its votes up
+        double top_item, top_cost;             // of one item of the largest tile, and of all of them with `more`
+        int32_t best_top;                      // the least top_cost from this cut on
+    };
+    int64_t n = 0, top = 32;  // rows; the largest tile
+    double least = 0.0;       // the shortest item there can be
+    int32_t count = 0;
+    Cut cut[40];
+
+    void form(const fp_device_forest *f, int64_t rows, int32_t max_R) {
+        const uint32_t nb = (uint32_t)f->hdr.n_bins;
+        n = rows;
+        top = std::min<int64_t>(max_R, (n + 31) / 32 * 32);
+        const int64_t tiles = n <= top ? 1 : (n + top - 1) / top;
+        for (uint32_t S = 1; count < 40; S = std::min(nb, S + 1 + S / 2)) {
+            const uint32_t bins = (nb + S - 1) / S;
+            Cut &c = cut[count++];
+            c.S = S;
+            c.fixed = item_cost(f, 0, bins);
+            c.per_row = item_cost(f, 1, bins) - c.fixed;
+            c.inv_row = 1.0 / c.per_row;
+            c.more = S > 1 ? 1000.0 : 0.0;
+            c.top_item = c.fixed + c.per_row * (double)top;
+            c.top_cost = (double)(tiles * S) * (c.top_item + c.more);
+            least = c.fixed + c.per_row * 32.0;
+            if (S == nb) break;
         }
-        if (S == nb) break;
+        for (int32_t i = count - 1; i >= 0; --i)
+            cut[i].best_top = i + 1 < count && cut[cut[i + 1].best_top].top_cost < cut[i].top_cost ? cut[i + 1].best_top : i;
     }
-    return best;
-}
+
+    // The shape when no item is to take longer than `most` nanoseconds: the
+    // splits whose items (as large as `most` lets them be) take the least time
+    // together.  *item: the time of one, *items: how many there are.
+    Shape within(double most, double *item, double *items) const {
+        Shape best;
+        auto take = [&](const Cut &c, int64_t R, double one, double cost) {
+            if (cost >= best.cost) return;
+            best.R = (int32_t)R;
+            best.S = (int32_t)c.S;
+            best.cost = cost;
+            *item = one;
+        };
+        for (int32_t i = 0; i < count; ++i) {
+            if (i > 0 && cut[i].top_item + cut[i].more <= most) {  // and so it is for more splits
+                const Cut &c = cut[cut[i].best_top];
+                take(c, top, c.top_item, c.top_cost);
+                break;
+            }
+            const Cut &c = cut[i];
+            int64_t R = top;
+            double one = c.top_item, cost = c.top_cost;
+            if (one > most) {
+                R = (int64_t)std::max(32.0, std::min((most - c.fixed) * c.inv_row, (double)top)) & ~(int64_t)31;
+                one = c.fixed + c.per_row * (double)R;
+                cost = (n <= R ? 1.0 : std::ceil((double)n / (double)R)) * (double)c.S * (one + c.more);
+            }
+            if (one + c.more > most) cost *= (one + c.more) / most;  // too long all the same: it counts for more
+            take(c, R, one, cost);
+        }
+        *items = std::ceil((double)n / best.R) * best.S;
+        return best;
+    }
+};
 
 // One persistent launch over up to FP_MAX_BATCH (forest, batch) pairs.  How
 // long an item may take is chosen for the whole launch: of a few lengths, the
@@ -1007,14 +1057,19 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
         max_R[m++] = R;
     }
     if (m == 0) return FP_OK;
-    double best_end = 1e300, most = 0.0;
+    BatchCuts cuts[FP_MAX_BATCH];
+    for (int32_t i = 0; i < m; ++i) cuts[i].form(forests[live[i]], batches[live[i]].n, max_R[i]);
+    Shape shapes[FP_MAX_BATCH], tried[FP_MAX_BATCH];
+    double best_end = 1e300, least = 0.0;  // the shortest item of some batch, which no shape undercuts
+    for (int32_t i = 0; i < m; ++i) least = std::max(least, cuts[i].least);
     for (double len = 8000.0; len < 4e6; len *= 1.5) {
+        if (len * 1.5 < least) continue;
         double sum = 0.0, longest = 0.0, items = 0.0;
+        bool whole = true;
         for (int32_t i = 0; i < m; ++i) {
-            const fp_device_forest *f = forests[live[i]];
-            const Shape sh = shape_within(f, batches[live[i]].n, max_R[i], len);
-            const double item = item_cost(f, sh.R, (f->hdr.n_bins + sh.S - 1) / sh.S);
-            const double count = (double)((batches[live[i]].n + sh.R - 1) / sh.R * sh.S);
+            double item = 0.0, count = 0.0;
+            tried[i] = cuts[i].within(len, &item, &count);
+            whole = whole && tried[i].S == 1 && tried[i].R == cuts[i].top;
             sum += item * count;
             items += count;
             longest = std::max(longest, item);
@@ -1022,8 +1077,9 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
         const double end = items <= sms ? longest : sum / sms + longest;
         if (end < best_end) {
             best_end = end;
-            most = len;
+            std::copy(tried, tried + m, shapes);
         }
+        if (whole) break;  // longer items there are none
     }
     size_t scratch_bytes = 256;  // the work counter, then per-batch accumulators and tile counters
     size_t acc_off[FP_MAX_BATCH] = {0}, cnt_off[FP_MAX_BATCH] = {0};
@@ -1033,7 +1089,7 @@ static int predict_batched_chunk(const fp_device_forest *const *forests, const f
         // one-word heads for every forest that has them, so that most launches
         // need one kind of walk (mixed kinds: 4 % longer)
         TravParams p = base_params(f, bt.X, bt.n, f->d_compact ? 3 : f->levels);
-        set_shape(p, shape_within(f, bt.n, max_R[i], most));
+        set_shape(p, shapes[i]);
         p.out_votes = bt.out_votes;
         p.out_class = bt.out_class;
         if (p.n_splits > 1) {
