@@ -41,7 +41,8 @@ struct fp_device_forest {
     int32_t nbuf = 3;                          // bin-block buffers
     size_t smem_votes = 0, smem_leaves = 0, smem_values = 0;
     int32_t grid_votes = 0, grid_leaves = 0, grid_values = 0;  // resident CTAs for a persistent launch
-    double cost_fixed = 0.0, cost_row = 0.0, cost_task = 0.0;  // of an item (fit_costs)
+    double cost_fixed = 0.0, cost_row = 0.0, cost_task = 0.0;  // of an item (fit_costs) ...
+    double cost_finish = 0.0;                                  // ... and, per row and thread, of a split tile's classes
     int32_t spin_limit = FP_SPIN_LIMIT;       // fault injection may lower it
     int32_t stall = 0;                        // fault injection: bin waits run out
 };
@@ -295,7 +296,11 @@ struct Part {
 //     heads are 4 levels);
 //   - its rows through one SM's loads;
 //   - its bins: 0.8 us in which the warps take their turn at a block, and its
-//     tasks, 0.06 ns per level in the head and 0.21 ns per level below it.
+//     tasks, 0.06 ns per level in the head and 0.21 ns per level below it;
+//   - the classes of a tile whose bins are split: the last CTA reads the votes
+//     of its rows anew, up to 32 lanes to a row, and every pass of its threads
+//     over them waits for L2, 1.1 us.  Without this term 9000 rows of a forest
+//     of 50 classes were split, 384 rows a tile: 68 us, 56 unsplit.
 void fit_costs(fp_device_forest *f) {
     const FpImageHeader &h = f->hdr;
     double levels = 1.0;  // of a tree's walk
@@ -304,6 +309,9 @@ void fit_costs(fp_device_forest *f) {
     f->cost_fixed = 4000.0 + 1000.0 * deep;
     f->cost_row = 0.08 * h.n_features;
     f->cost_task = h.n_super ? 0.3 + 0.06 * head + 0.21 * deep : 0.06 * head;
+    int lanes = 1;
+    while (lanes < h.n_classes && lanes < 32) lanes *= 2;
+    f->cost_finish = h.n_values > 0 ? 0.0 : 1100.0 * lanes;
 }
 
 double item_cost(const fp_device_forest *f, int64_t R, int64_t bins) {
@@ -312,8 +320,12 @@ double item_cost(const fp_device_forest *f, int64_t R, int64_t bins) {
 }
 
 // The best shape for n rows, fewer than a few waves' worth: in one split if
-// `whole` allows it, in several (up to one per bin) if `split` does and saves
-// a fifth; `extra`: what splitting costs besides.
+// `whole` allows it, in several (up to one per bin) if `split` does.  `extra`:
+// what splitting costs the GPU besides, where the splits add up in scratch.
+// The host's part of such a call is 6 us longer (the allocation, the memset
+// and the counters), which bounds small calls that follow one another, so it
+// has to be saved as well, and 15 % of the estimate at least (256 shallow
+// trees, 1000 rows: 21 us a call split, 17.5 unsplit).
 Shape best_shape(const fp_device_forest *f, int64_t n, int32_t slots, bool whole, bool split, double extra) {
     const int32_t nb = f->hdr.n_bins;
     Shape best;
@@ -323,7 +335,8 @@ Shape best_shape(const fp_device_forest *f, int64_t n, int32_t slots, bool whole
             const int64_t fit = ((n + w * room - 1) / (w * room) + 31) / 32 * 32;
             const int64_t R = std::min<int64_t>(f->R, std::max<int64_t>(32, fit));
             const int64_t tiles = (n + R - 1) / R, turns = (tiles + room - 1) / room;
-            const double c = (double)turns * item_cost(f, R, (nb + S - 1) / S) + (S > 1 ? extra : 0.0);
+            double c = (double)turns * item_cost(f, std::min(n, R), (nb + S - 1) / S);
+            if (S > 1 && extra > 0.0) c += extra + f->cost_finish * (double)R / f->threads;
             if (c < best.cost) {
                 best.R = (int32_t)R;
                 best.S = (int32_t)S;
@@ -338,7 +351,7 @@ Shape best_shape(const fp_device_forest *f, int64_t n, int32_t slots, bool whole
         for (int64_t S = 2; S < nb && S <= slots; S += 1 + S / 6) try_splits(S);
         if (nb > 1) try_splits(nb);
     }
-    if (whole && extra > 0.0 && best.cost > 0.8 * unsplit.cost) return unsplit;
+    if (whole && extra > 0.0 && best.cost > std::min(0.85 * unsplit.cost, unsplit.cost - 6000.0)) return unsplit;
     return best;
 }
 
