@@ -335,7 +335,9 @@ Shape best_shape(const fp_device_forest *f, int64_t n, int32_t slots, bool whole
             const int64_t fit = ((n + w * room - 1) / (w * room) + 31) / 32 * 32;
             const int64_t R = std::min<int64_t>(f->R, std::max<int64_t>(32, fit));
             const int64_t tiles = (n + R - 1) / R, turns = (tiles + room - 1) / room;
-            double c = (double)turns * item_cost(f, std::min(n, R), (nb + S - 1) / S);
+            // a slab of few rows is walked by as many warp steps in the heads, fewer below them
+            const int64_t filled = n < R ? (n + R) / 2 : R;
+            double c = (double)turns * item_cost(f, filled, (nb + S - 1) / S);
             if (S > 1 && extra > 0.0) c += extra + f->cost_finish * (double)R / f->threads;
             if (c < best.cost) {
                 best.R = (int32_t)R;
