@@ -33,7 +33,8 @@
 // 0xFFFFFFFF and a NaN threshold to 0.  For every observation value x and
 // threshold t, x <= t (go left) exactly when key(x) <= key(t) -- a NaN x or t
 // goes right, as the float compare does -- so the kernel converts the rows
-// once when it stages them and every compare is an unsigned integer compare.
+// once when it stages them and every compare is an unsigned integer compare
+// (it stages one less than the key, and x <= t is staged x < key(t)).
 //
 // Super-nodes of format 2 (below) compare remapped keys, which spread the
 // forest's own thresholds over the word.  First the widest run of keys that
@@ -52,7 +53,7 @@
 // (above top) below (above) every threshold; the shift is one-to-one.  So x
 // <= t exactly when V(key(x)) <= V(key(t)).  A NaN threshold and a dummy slot
 // store 0, below every V(key(x)) (remapped, every row value has the top bit
-// set), so every x goes right of them.  Rows are staged as V(key(x)) and
+// set), so every x goes right of them.  Rows are staged as V(key(x)) - 1 and
 // every stored threshold, in the heads too, is V(key(t)).  Short prefixes of
 // V distinguish the forest's thresholds far better than prefixes of the key,
 // whose top bits spend themselves on the sign and on exponents that no
@@ -130,7 +131,7 @@
 //           the super-nodes rooted at its internal exits are consecutive, in
 //           exit order, so exit e continues at this + offset + (number of
 //           internal exits before e)
-// The first two levels compare full keys; the last compares the key of x
+// The first two levels compare full keys; the last compares the staged x
 // with a key prefix, and when the prefixes are equal it decides with the full
 // key from deep_keys (a 4-byte load, for a small fraction of compares).  A
 // dummy slot has key 0 (every observation goes right of it, never a tie).
@@ -141,7 +142,7 @@
 //   w[3..6] slots 3..6: [fb-1:0] feature, [fb+cb-1:fb] class of the left exit,
 //           [fb+2cb-1:fb+cb] of the right one, [31:fb+2cb] the top bits of V
 //   w[7]    as in format 1
-// A staged V(key(x)) compared with the whole word decides the split wherever
+// A staged V(key(x)) - 1 compared with the whole word decides the split wherever
 // its top bits differ from the slot's prefix; where they are equal (rare: the
 // forest's thresholds are spread over the prefix range) the slot's full V
 // from deep_keys decides.  Dummy slots and NaN thresholds store V = 0, whose

@@ -176,18 +176,24 @@ __device__ __forceinline__ uint32_t remap_key(const TravParams &p, uint32_t k) {
     return p.kflag | ((min(max(g, p.klo), p.khi) - p.klo) << p.kshl);
 }
 
-// A staged observation value for super-node kind DK: its float bits (2), its
-// order key (3) or its remapped key (4).
+// A staged observation value for super-node kind DK: its float bits (2), or
+// one less than its order key (3) or remapped key (4; no key is 0).  One less,
+// so that a value equal to a threshold, as rows of whole numbers or of few
+// distinct values have, shares no prefix with it where the bits below are
+// zero: prefixes that are equal cost a look at the full keys (64 trees on 28
+// binary features with thresholds on their values, 200,000 rows: 190 us, 327
+// with the keys themselves).
 template <int DK>
 __device__ __forceinline__ uint32_t staged(const TravParams &p, float v) {
-    return DK == 2 ? __float_as_uint(v) : (DK == 3 ? obs_key(v) : remap_key(p, obs_key(v)));
+    return DK == 2 ? __float_as_uint(v) : (DK == 3 ? obs_key(v) : remap_key(p, obs_key(v))) - 1u;
 }
 
-// x <= t, the split's test (go left): keys compare as unsigned integers,
-// otherwise as floats (a NaN x or t goes right either way).
+// x <= t, the split's test (go left): keys compare as unsigned integers (the
+// staged x being one less), otherwise as floats (a NaN x or t goes right either
+// way).
 template <bool KEYS>
 __device__ __forceinline__ bool goes_left(uint32_t x, uint32_t t) {
-    return KEYS ? x <= t : __uint_as_float(x) <= __uint_as_float(t);
+    return KEYS ? x < t : __uint_as_float(x) <= __uint_as_float(t);
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -379,13 +385,13 @@ __device__ __forceinline__ DeepStep deep_step3(const TravParams &p, uint32_t ref
                                                const uint32_t w[8]) {
     const uint32_t fm7 = p.fmask << 7;
     const uint32_t k0 = lds(xb + (__funnelshift_r(w[3], w[3], p.frot) & fm7));
-    const bool r0 = k0 > w[0];
+    const bool r0 = k0 >= w[0];
     const uint32_t n1 = r0 ? w[2] : w[1], m1 = r0 ? w[5] : w[4];
     const uint32_t k1 = lds(xb + (__funnelshift_r(m1, m1, p.frot) & fm7));
-    const bool r1 = k1 > n1;
+    const bool r1 = k1 >= n1;
     const uint32_t n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
     const uint32_t k2 = lds(xb + ((n2 & p.fmask) << 7));
-    bool r2 = k2 > n2;  // decided by the key bits, unless they are equal
+    bool r2 = k2 >= n2;  // decided by the key bits, unless they are equal
     DeepStep s;
     s.e = (r0 ? 4u : 0u) + (r1 ? 2u : 0u);
     // behind a vote, so that the steps without a tie issue no load of the side
@@ -393,7 +399,7 @@ __device__ __forceinline__ DeepStep deep_step3(const TravParams &p, uint32_t ref
     // a wavefront a step (2 % of the run)
     const bool tie = (k2 ^ n2) < p.tie && ref != FP_NO_TASK;
     if (__any_sync(0xffffffffu, tie)) {
-        if (tie) r2 = k2 > __ldg(p.deep_keys + 4 * (int64_t)ref + (s.e >> 1));
+        if (tie) r2 = k2 >= __ldg(p.deep_keys + 4 * (int64_t)ref + (s.e >> 1));
         __syncwarp();
     }
     s.e += r2 ? 1u : 0u;
@@ -411,25 +417,25 @@ __device__ __forceinline__ DeepStep deep_step3p(const TravParams &p, uint32_t re
                                                 const uint32_t w[8]) {
     const uint32_t fm = p.fmask;
     const uint32_t k0 = lds(xb + ((w[0] & fm) << 7));
-    bool r0 = k0 > w[0];
+    bool r0 = k0 >= w[0];
     uint32_t n1 = r0 ? w[2] : w[1];
     const uint32_t k1 = lds(xb + ((n1 & fm) << 7));
-    bool r1 = k1 > n1;
+    bool r1 = k1 >= n1;
     uint32_t n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
     uint32_t k2 = lds(xb + ((n2 & fm) << 7));
-    bool r2 = k2 > n2;
+    bool r2 = k2 >= n2;
     // one test for the three slots, by the last level's shorter prefix: it
     // takes a few more steps again than need be
     const bool tie = min(min(k0 ^ w[0], k1 ^ n1), k2 ^ n2) < p.tie && ref != FP_NO_TASK;
     if (__any_sync(0xffffffffu, tie)) {
         if (tie) {
             const uint32_t *fk = p.deep_keys + 8 * (int64_t)ref;
-            r0 = k0 > __ldg(fk);
+            r0 = k0 >= __ldg(fk);
             n1 = r0 ? w[2] : w[1];
-            r1 = lds(xb + ((n1 & fm) << 7)) > __ldg(fk + 1 + (r0 ? 1 : 0));
+            r1 = lds(xb + ((n1 & fm) << 7)) >= __ldg(fk + 1 + (r0 ? 1 : 0));
             n2 = r0 ? (r1 ? w[6] : w[5]) : (r1 ? w[4] : w[3]);
             k2 = lds(xb + ((n2 & fm) << 7));
-            r2 = k2 > __ldg(fk + 3 + (r0 ? 2 : 0) + (r1 ? 1 : 0));
+            r2 = k2 >= __ldg(fk + 3 + (r0 ? 2 : 0) + (r1 ? 1 : 0));
         }
         __syncwarp();
     }
@@ -503,14 +509,14 @@ __device__ __noinline__ uint32_t packed_walk(const TravParams &p, int b, int k, 
     if (p.packed_kind == 2) {
         for (int l = 0; l <= p.depth; l += 2) {
             const uint4 nd = __ldg(reinterpret_cast<const uint4 *>(blk) + q * bn.stride + k);
-            const bool r0 = lds(xb + ((nd.w & 1023u) << 7)) > nd.x;
-            const bool r1 = lds(xb + (((nd.w >> (r0 ? 20 : 10)) & 1023u) << 7)) > (r0 ? nd.z : nd.y);
+            const bool r0 = lds(xb + ((nd.w & 1023u) << 7)) >= nd.x;
+            const bool r1 = lds(xb + (((nd.w >> (r0 ? 20 : 10)) & 1023u) << 7)) >= (r0 ? nd.z : nd.y);
             q = 4u * q + 1u + (r0 ? 2u : 0u) + (r1 ? 1u : 0u);
         }
     } else {
         for (int l = 0; l <= p.depth; ++l) {
             const uint2 nd = __ldg(reinterpret_cast<const uint2 *>(blk) + q * bn.stride + k);
-            q = 2u * q + 1u + (lds(xb + ((nd.y >> 22) << 7)) > nd.x ? 1u : 0u);
+            q = 2u * q + 1u + (lds(xb + ((nd.y >> 22) << 7)) >= nd.x ? 1u : 0u);
         }
     }
     return q - (uint32_t)bn.nranks;
@@ -540,15 +546,15 @@ __device__ __forceinline__ uint32_t head_walk(const TravParams &p, int b, uint32
 #pragma unroll 1  // two levels a turn: one saves loop control (1 % of the run), five or ten no more
         for (int l = p.depth; l > 0; l -= 2) {
             const uint32_t na = lds(at), xa = lds(xb + ((na & p.fmask) << 7));
-            at = 2u * at + (xa > na ? right : left);
+            at = 2u * at + (xa >= na ? right : left);
             const uint32_t nb = lds(at), x2 = lds(xb + ((nb & p.fmask) << 7));
             near = min(near, min(xa ^ na, x2 ^ nb));
-            at = 2u * at + (x2 > nb ? right : left);
+            at = 2u * at + (x2 >= nb ? right : left);
         }
         if (!(p.depth & 1)) {
             const uint32_t nd = lds(at), x = lds(xb + ((nd & p.fmask) << 7));
             near = min(near, x ^ nd);
-            at = 2u * at + (x > nd ? right : left);
+            at = 2u * at + (x >= nd ? right : left);
         }
         const bool tie = my && near <= p.fmask;  // the top bits were equal somewhere (rare)
         if (__any_sync(0xffffffffu, tie)) {
