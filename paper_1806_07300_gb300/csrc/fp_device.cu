@@ -31,6 +31,7 @@ struct fp_device_forest {
     uint8_t *d_compact = nullptr;  // one-word level heads, after their bins (NULL: none)
     int64_t compact_bins_bytes = 0;
     int32_t *d_status = nullptr;
+    int64_t l2_bytes = 0;     // of the device's L2
     int32_t R = 0;            // observation tile actually launched (fits shared memory)
     int32_t threads = 0;
     int32_t refill = 8;
@@ -365,10 +366,13 @@ int plan_rows(const fp_device_forest *f, int64_t n, int32_t grid, bool split, bo
     const int64_t wave = (int64_t)grid * f->R;  // rows of a full wave of the largest tiles
     const bool passes = h.n_passes > 1;
     // A forest beyond L2 whose tiles are too small to use a bin's lines before
-    // the next bin's evict them (more than 16 bytes of it per task in a wave)
-    // is swept pass by pass, all tiles of a pass before the next pass.
+    // the next bin's evict them is swept pass by pass, all tiles of a pass
+    // before the next pass.  256 trees of 208 MB, 400,000 rows: 11.1 ms by
+    // passes, 12.3 in one sweep with 32-row tiles (167 bytes of the forest per
+    // task of a wave), 6.22 and 6.45 with 64 rows (83 bytes), 4.10 and 3.87
+    // with 128; in two to four waves (20,000 rows) one sweep is the faster.
     const int64_t deep = 32 * (int64_t)h.n_super;
-    if (passes && deep > ((int64_t)96 << 20) && deep > 16 * wave * h.n_trees) {
+    if (passes && deep > f->l2_bytes / 4 * 3 && deep > 64 * wave * h.n_trees && n >= 8 * wave) {
         const int64_t want = (n * h.n_passes + grid - 1) / grid;
         out[0].row0 = 0;
         out[0].n = n;
@@ -602,9 +606,12 @@ extern "C" int fp_upload(const fp_packed_forest *pf, void *stream, fp_device_for
     f->passes.assign(reinterpret_cast<const FpPass *>(img + h->off_passes),
                      reinterpret_cast<const FpPass *>(img + h->off_passes) + h->n_passes);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    int rc = FP_OK;
+    int rc = FP_OK, l2 = 0;
     cudaError_t e = cudaGetDevice(&f->device);
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaGetDevice"); goto fail; }
+    e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, f->device);
+    if (e != cudaSuccess) { rc = cuda_fail(e, "cudaDeviceGetAttribute"); goto fail; }
+    f->l2_bytes = l2;
     if (injected_alloc_failure("cudaMalloc(image)")) { rc = FP_ENOMEM; goto fail; }
     e = cudaMalloc(&f->d_image, (size_t)h->total_bytes);
     if (e != cudaSuccess) { rc = cuda_fail(e, "cudaMalloc(image)"); goto fail; }
