@@ -156,14 +156,14 @@ void (*traverse_kernel(const fp_device_forest *f))(TravParams) {
 }
 
 // Every instance of the batched kernel: super-node kind (0 mixed, 2, 3, 4) x
-// head kind (-1 mixed, 0 ranked, 1, 2, 3).
+// head kind (-1 mixed, 0 ranked, 1, 2, 3; two-level forests have no one-word heads).
 template <int KIND>
 void add_batched(std::vector<void (*)(BatchParams)> &v) {
     v.push_back(fp_traverse_batched_kernel<KIND, -1>);
     v.push_back(fp_traverse_batched_kernel<KIND, 0>);
     v.push_back(fp_traverse_batched_kernel<KIND, 1>);
     v.push_back(fp_traverse_batched_kernel<KIND, 2>);
-    v.push_back(fp_traverse_batched_kernel<KIND, 3>);
+    v.push_back(fp_traverse_batched_kernel<KIND, KIND == 2 ? -1 : 3>);
 }
 
 const std::vector<void (*)(BatchParams)> &batched_kernels() {

@@ -1322,7 +1322,7 @@ struct BatchParams {
 
 // KIND: 2, 3 or 4 when every forest of the launch has that kind of
 // super-node (one walk compiled in), 0 for a mix (all, chosen per item).  HK:
-// the head kind when all forests share it (0 ranked, 1, 2), else -1.
+// the head kind when all forests share it (0 ranked, 1, 2, 3), else -1.
 template <int KIND, int HK>
 __global__ void __launch_bounds__(1024, 1) fp_traverse_batched_kernel(const __grid_constant__ BatchParams bp) {
     extern __shared__ __align__(16) uint8_t smem[];
