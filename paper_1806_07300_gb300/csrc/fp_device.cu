@@ -323,10 +323,10 @@ double item_cost(const fp_device_forest *f, int64_t R, int64_t bins) {
 // The best shape for n rows, fewer than a few waves' worth: in one split if
 // `whole` allows it, in several (up to one per bin) if `split` does.  `extra`:
 // what splitting costs the GPU besides, where the splits add up in scratch.
-// The host's part of such a call is 6 us longer (the allocation, the memset
-// and the counters), which bounds small calls that follow one another, so it
-// has to be saved as well, and 15 % of the estimate at least (256 shallow
-// trees, 1000 rows: 21 us a call split, 17.5 unsplit).
+// The allocation, the memset and their place between kernels add 3 to 6 us to
+// small calls that follow one another, so as much has to be saved as well, and
+// 15 % of the estimate at least (256 shallow trees, 1000 rows: 21 us a call
+// split, 17.5 unsplit).
 Shape best_shape(const fp_device_forest *f, int64_t n, int32_t slots, bool whole, bool split, double extra) {
     const int32_t nb = f->hdr.n_bins;
     Shape best;
@@ -514,6 +514,16 @@ bool may_split(cudaStream_t s) {
     return false;
 }
 
+// plan_rows for a call that takes scratch where bins of a forest of one pass
+// are split.  The stream is asked only then: most calls split nothing (a call
+// of 32 rows of 16 trees takes the host 2.22 us, 2.34 when it asks, and 4.7
+// where bins are split).
+int plan_call(const fp_device_forest *f, int64_t n, int32_t grid, cudaStream_t s, Part out[2]) {
+    int k = plan_rows(f, n, grid, true, false, out);
+    if (f->hdr.n_passes == 1 && out[k - 1].shape.S > 1 && !may_split(s)) k = plan_rows(f, n, grid, false, false, out);
+    return k;
+}
+
 // Scratch of a part whose splits add up in global memory: acc_per_row bytes of
 // accumulator per row, then a counter per tile.
 size_t scratch_bytes(const Part &pt, int64_t acc_per_row, size_t *acc_bytes) {
@@ -674,17 +684,19 @@ namespace {
 
 // fp_predict and fp_predict_noalloc: scratch_for(bytes, &ptr) supplies the
 // scratch of a part, release(ptr) takes it back.  A part that gets none runs
-// unsplit where the forest has one pass, or where `whole` says so.  Votes
+// unsplit where the forest has one pass, or where `whole` says so (then a
+// forest of one pass is not split at all).  Votes
 // without classes take no scratch: the splits add up in the caller's votes and
 // nothing is left to do after the last of them.  So such calls cannot fail for
 // memory, put no memory node into a captured graph, and overlap freely when
 // they are fp_predict_noalloc's.
 template <class Scratch, class Release>
 int predict_votes(const fp_device_forest *f, const float *X, int64_t n, uint32_t *out_votes, int32_t *out_class,
-                  cudaStream_t s, bool split, bool whole, Scratch scratch_for, Release release) {
+                  cudaStream_t s, bool whole, Scratch scratch_for, Release release) {
     const FpImageHeader &h = f->hdr;
     Part parts[2];
-    const int k = plan_rows(f, n, f->grid_votes, split, false, parts);
+    const int k = whole || !out_class ? plan_rows(f, n, f->grid_votes, !whole, false, parts)
+                                      : plan_call(f, n, f->grid_votes, s, parts);
     for (int i = 0; i < k; ++i) {
         Part &pt = parts[i];
         uint32_t *const votes = out_votes ? out_votes + pt.row0 * h.n_classes : nullptr;
@@ -737,7 +749,7 @@ extern "C" int fp_predict(const fp_device_forest *f, const float *X, int64_t n, 
     if (rc) return rc;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     return predict_votes(
-        f, X, n, out_votes, out_class, s, !out_class || may_split(s), false,
+        f, X, n, out_votes, out_class, s, false,
         [&](size_t bytes, void **out) { return scratch_alloc(f->device, out, bytes, s); },
         [&](void *ptr) { cudaFreeAsync(ptr, s); });
 }
@@ -758,7 +770,7 @@ extern "C" int fp_predict_values(const fp_device_forest *f, const float *X, int6
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const FpImageHeader &h = f->hdr;
     Part parts[2];
-    const int k = plan_rows(f, n, f->grid_values, may_split(s), false, parts);
+    const int k = plan_call(f, n, f->grid_values, s, parts);
     for (int i = 0; i < k; ++i) {
         Part &pt = parts[i];
         size_t acc_bytes;  // a float accumulator per row, a counter per tile
@@ -852,7 +864,7 @@ extern "C" int fp_predict_noalloc(const fp_device_forest *f, const float *X, int
         if (rc) return rc;
     }
     return predict_votes(
-        f, X, n, out_votes, out_class, s, false, true,
+        f, X, n, out_votes, out_class, s, true,
         [&](size_t bytes, void **out) {
             if (bytes > FP_NOALLOC_SCRATCH_BYTES) {
                 fp_set_error("fp_predict_noalloc: %zu bytes of scratch, more than the fixed %u", bytes,
