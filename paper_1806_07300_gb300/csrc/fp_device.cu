@@ -43,6 +43,7 @@ struct fp_device_forest {
     size_t smem_votes = 0, smem_leaves = 0, smem_values = 0;
     int32_t grid_votes = 0, grid_leaves = 0, grid_values = 0;  // resident CTAs for a persistent launch
     double cost_fixed = 0.0, cost_row = 0.0, cost_task = 0.0;  // of an item (fit_costs) ...
+    double deep_levels = 0.0;                                  // of a tree's walk, below the heads (fit_costs)
     double cost_finish = 0.0;                                  // ... and, per row and thread, of a split tile's classes
     int32_t spin_limit = FP_SPIN_LIMIT;       // fault injection may lower it
     int32_t stall = 0;                        // fault injection: bin waits run out
@@ -307,6 +308,7 @@ void fit_costs(fp_device_forest *f) {
     double levels = 1.0;  // of a tree's walk
     for (int64_t m = h.n_internal / std::max<int32_t>(1, h.n_trees); m > 1; m >>= 1) levels += 1.4;
     const double head = std::min(levels, h.depth + 1.0), deep = h.n_super ? levels - head : 0.0;
+    f->deep_levels = deep;
     f->cost_fixed = 4000.0 + 1000.0 * deep;
     f->cost_row = 0.08 * h.n_features;
     f->cost_task = h.n_super ? 0.3 + 0.06 * head + 0.21 * deep : 0.06 * head;
@@ -454,6 +456,7 @@ TravParams base_params(const fp_device_forest *f, const float *X, int64_t n, int
     p.n_vals = (uint32_t)h.n_values;
     p.depth = h.depth;
     p.refill = f->refill;
+    p.step_bins = f->deep_levels >= 10.0;  // measured on both sides: 8 levels lose 12 %, 13 gain 15 %
     p.status = f->d_status;
     p.spin_limit = f->spin_limit;
     p.stall = f->stall;
