@@ -3,10 +3,12 @@
 // fp_upload copies a packed image to the device; fp_predict launches the
 // persistent traversal kernel (fp_traverse.cuh) on the caller's stream, in the
 // shape that plan_rows chooses for the batch.  The kernel needs scratch memory
-// only where a forest of several passes has its bins split over CTAs (a vote
-// accumulator when the caller asks for classes only, and one counter per
-// observation tile); that scratch comes from a library-owned stream-ordered
-// memory pool, so calls on different streams never share it.
+// only where bins are split over CTAs and more than votes is asked for: one
+// counter per observation tile, and an accumulator (of votes, unless they add
+// up in the caller's buffer; of leaf values).  Bins of a forest of one pass are
+// not split for it under capture or in fp_predict_noalloc.  The scratch comes
+// from a library-owned stream-ordered memory pool, so calls on different
+// streams never share it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -127,7 +129,11 @@ void (*traverse_kernel_sized(const fp_device_forest *f))(TravParams) {
 // level slots of one word).
 template <int MODE, int DK>
 void (*traverse_kernel_deep(const fp_device_forest *f))(TravParams) {
-    if (f->hdr.n_super == 0) {  // one build serves every CTA size
+    // Shallow forests: one build for every CTA size.  Its 39 to 64 registers
+    // keep a second CTA of 24 warps, or a third of 16, off the SM, and the large
+    // CTA is the fastest all the same (256 boosted trees, 1 M rows: 580 us with
+    // 32 warps, 615 with 24, 616 to 656 with 16).
+    if (f->hdr.n_super == 0) {
         switch (f->levels) {
             case 1: return fp_traverse_kernel<MODE, 1, DK, 1, true>;
             case 2: return fp_traverse_kernel<MODE, 1, DK, 2, true>;
@@ -805,10 +811,10 @@ extern "C" int fp_predict_values(const fp_device_forest *f, const float *X, int6
 
 // ---------------------------------------------------------------------------
 // fp_predict_noalloc: fp_predict for callers that must not allocate device
-// memory.  The scratch that a forest swept in several passes needs (a vote
-// accumulator when no votes buffer is given, one counter per observation
-// tile when classes are asked for) lives in this fixed array instead of the
-// stream-ordered pool.  Every GPU that loads the library holds the array
+// memory.  The scratch of a forest of several passes whose bins are split and
+// whose classes are asked for (one counter per observation tile, and a vote
+// accumulator unless the votes add up in a buffer of the caller's of more than
+// 4 MiB) lives in this fixed array instead of the stream-ordered pool.  Every GPU that loads the library holds the array
 // until the process exits.
 #define FP_NOALLOC_SCRATCH_BYTES (16u << 20)
 static __device__ __align__(256) unsigned char fp_noalloc_scratch[FP_NOALLOC_SCRATCH_BYTES];
