@@ -411,6 +411,28 @@ def tuned_forest(args, forest, X, name):
     return df, tuning
 
 
+def kernels_per_call(call, stream) -> int:
+    """Kernels that one call launches on the stream, counted in a captured
+    graph of it (a batch of some waves and a rest is two launches)."""
+    import ctypes
+    import torch
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=stream):
+        call()
+    drv, graph, n = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t(0)
+    if drv.cuGraphGetNodes(graph, None, ctypes.byref(n)):
+        raise RuntimeError("cuGraphGetNodes failed")
+    nodes = (ctypes.c_void_p * n.value)()
+    if drv.cuGraphGetNodes(graph, nodes, ctypes.byref(n)):
+        raise RuntimeError("cuGraphGetNodes failed")
+    kernels, kind = 0, ctypes.c_int()
+    for node in nodes:
+        if drv.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)):
+            raise RuntimeError("cuGraphNodeGetType failed")
+        kernels += kind.value == 0  # CU_GRAPH_NODE_TYPE_KERNEL
+    return kernels
+
+
 def run_packed(args, ws, rank, local):
     import torch
     import datagen
@@ -456,7 +478,7 @@ def run_packed(args, ws, rank, local):
     time.sleep(0.3)
     barrier()
     torch.cuda.synchronize()
-    # the timed region: K steps, one launch each, back to back on the stream
+    # the timed region: K steps, one call each, back to back on the stream
     # (inputs larger than L2), or each after an L2 flush and timed alone
     total_ms, per_launch_ms = timed_steps(lambda: step(X, votes, cls, stream), args.steps, stream, flush)
     barrier()
@@ -609,7 +631,7 @@ def run_packed(args, ws, rank, local):
         "plain_baseline": plain,
         "packed_vs_plain": (value / ws / plain["value"]) if plain else None,
         "e2e": e2e,
-        "gpu_launches": args.steps,  # at least: a call of some waves and a tail is two launches
+        "gpu_launches": args.steps * kernels_per_call(lambda: step(X, votes, cls, stream), stream),
         # single launches timed one by one after the timed region: median and spread
         "launch_ms": {"median": statistics.median(per_launch_ms), "min": min(per_launch_ms),
                       "max": max(per_launch_ms), "n": len(per_launch_ms)},

@@ -55,12 +55,11 @@
 // last split's CTA writes it).
 //
 // What bounds it (256 trees of 78.8k nodes, 28 features, 4 M rows, bins of 5
-// trees with heads 0..9: 24.0 ms; 27.5 ms as one pass of L2 after another with
-// steps of divergent branches): the load/store data pipe, 80 % busy with 6.2
-// wavefronts per (row, tree), a little over half of them the super-nodes'
-// sectors and the rest shared-memory words; 17.9 warp instructions per (row,
-// tree) (23.4 before) take 63 % of the issue slots.  (Counters of the walk at
-// 24.4 ms, before level heads of one word per node.)
+// trees with heads 0..9: 24.1 ms; 27.5 ms as one pass of L2 after another with
+// steps of divergent branches): the load/store data pipe, 77 % busy with 5.7
+// wavefronts per (row, tree), 4.5 sectors of super-nodes and rows and 2.5
+// wavefronts of shared memory among them (6.3 before); 18.7 warp instructions
+// per (row, tree) (23.4 before) take 63 % of the issue slots.
 //
 // Waits: __syncthreads is a hardware wait; a wait for
 // a bin block polls its mbarrier at most spin_limit times (FP_SPIN_LIMIT
